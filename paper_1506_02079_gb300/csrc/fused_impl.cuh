@@ -23,7 +23,7 @@
 //
 // Coarse tail (k_tail).  Levels whose larger side is <= 64 are run by one CTA per slice: the
 // remaining down and up legs of the V-cycle with __syncthreads() between half-sweeps, on
-// L1-resident data.  Same per-cell arithmetic as every other schedule.
+// copies in shared memory.  Same per-cell arithmetic as every other schedule.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -674,124 +674,262 @@ __global__ void __launch_bounds__(kWaveWarps * 32, WaveOcc<T, S>::value) k_wave(
 
 // ---------------------------------------------------------------- coarse tail
 // The levels of one slice from kc (the first with both sides <= kTailMax) down to 1 x 1 are run
-// by one CTA on copies in shared memory (dense rows): at most 64 x 64 + 32 x 32 + ... cells, u and
-// b each.  Only level kc touches global memory: its right-hand side (and, continuing at level 0,
-// its iterate) is read at the start and its final iterate written at the end, where the wavefront
-// UP kernel of level kc - 1 (or the residual kernel, at kc = 0) reads it.  The per-cell arithmetic
-// and its order are those of every other schedule.
+// by one CTA on copies in shared memory: at most 64 x 64 + 32 x 32 + ... cells, u and b each.
+// Only level kc touches global memory: its right-hand side (and, continuing at level 0, its
+// iterate) is read at the start and its final iterate written at the end, where the wavefront
+// UP kernel of level kc - 1 (or the residual kernel, at kc = 0) reads it.  The per-cell
+// arithmetic and its order are those of every other schedule.
+//
+// Bound by the latency of about 70 dependent passes (half-sweeps, restrictions, prolongations)
+// over few cells, so each pass is kept short: the iterate has a border of zeros (no range checks:
+// a missing neighbour has coefficient 0), the stencils come from a table of the at most 4 x 4
+// different ones of a level (first, inner, last but one and last cell of each axis), the
+// interpolation weights from tables, a thread loads the inputs of up to four cells before it
+// stores any, and levels of at most 8 x 8 cells are run by one warp without block barriers.
+// 64 slices of 64 x 64, 2 + 2 sweeps: 137 -> 35 us per launch against stencils formed per cell and
+// pass, which took most of the instructions; the finest level is now bound by shared-memory
+// bandwidth (two-way conflicts of the stride-2 accesses), the small ones by latency.
+constexpr int kTailMaxLevels = 16;
+constexpr int kTailThreads = 512;
+
+// One of the stencils of a level, 16-byte aligned for vector loads.
 template <class T>
-__device__ void tail_relax(const LSlice<T>& L, int k, T alpha, T sk, int sweeps) {
-    const int n = L.nx * L.ny;
-    for (int s = 0; s < sweeps; ++s)
-        for (int color = 0; color < 2; ++color) {
-            for (int p = threadIdx.x; p < n; p += blockDim.x) {
-                const int y = p / L.nx, x = p - y * L.nx;
-                if (((x + y) & 1) != color) continue;
-                const Coef<T> c = coef_at<T>(x, y, L.nx, L.ny, L.n0x, L.n0y, k, alpha, sk);
-                const int64_t q = (int64_t)y * L.pitch + x;
-                const T uw = x > 0 ? L.u[q - 1] : T(0);
-                const T ue = x + 1 < L.nx ? L.u[q + 1] : T(0);
-                const T un = y > 0 ? L.u[q - L.pitch] : T(0);
-                const T us = y + 1 < L.ny ? L.u[q + L.pitch] : T(0);
-                L.u[q] = gs_update<T>(c, L.b[q], uw, ue, un, us);
-            }
-            __syncthreads();
-        }
+struct alignas(16) TailCoef {
+    T cw, ce, cn, cs, iD, D, pad0, pad1;
+};
+
+template <class T>
+__device__ __forceinline__ Coef<T> tail_coef(const TailCoef<T>* t) {
+    Coef<T> c;
+    T q[4];
+    Vec4<T>::load(&t->cw, q);
+    c.cw = q[0]; c.ce = q[1]; c.cn = q[2]; c.cs = q[3];
+    Vec2<T>::load(&t->iD, c.iD, c.D);
+    return c;
 }
 
-constexpr int kTailMaxLevels = 16;
+// Class of index i of an axis of n cells: 0 first, 1 inner (all three cells full), 2 last but one,
+// 3 last; axis_coef is the same for all inner cells.
+__device__ __forceinline__ int tail_class(int i, int n) {
+    return i >= 1 && i + 2 < n ? 1 : (i == 0 ? 0 : (i == n - 1 ? 3 : 2));
+}
 
 template <class T>
-__global__ void __launch_bounds__(512) k_tail(TailArgs<T> a) {
+struct TailLevel {
+    T* u;        // cell (0, 0) of the bordered iterate (row pitch nx + 2)
+    T* b;        // right-hand side (row pitch nx)
+    const TailCoef<T>* coef;  // [class of y][class of x]
+    const T *wx, *wy;         // interpolation weights of this level's cells toward J
+    const signed char *jx, *jy;  // J - I along each axis (0, -1 or 1)
+    int nx, ny;
+};
+
+// Where a level's arrays start in the CTA's shared memory (offsets, not pointers, so that the
+// accesses stay shared-memory ones).
+struct TailOffsets {
+    int u, b, x, y, nx, ny;
+};
+
+// `threads` threads (a power of two) on the cells of one colour: 2^sh lanes across the row.
+__device__ __forceinline__ int tail_shift(int cells_x, int threads) {
+    int sh = 0;
+    while ((1 << sh) < cells_x && (1 << sh) < 32 && (1 << sh) < threads) ++sh;
+    return sh;
+}
+
+template <class T, class Sync>
+__device__ __forceinline__ void tail_relax(const TailLevel<T>& L, int sweeps, int tid, int threads, Sync sync) {
+    const int nx = L.nx, ny = L.ny, pu = nx + 2;
+    const int sh = tail_shift((nx + 1) >> 1, threads);
+    const int lx = tid & ((1 << sh) - 1), ly = tid >> sh, rows = threads >> sh;
+    constexpr int B = 4;  // cells in flight per thread
+    for (int h = 0; h < 2 * sweeps; ++h) {
+        for (int y0 = ly; y0 < ny; y0 += B * rows) {
+            T v[B];
+#pragma unroll
+            for (int i = 0; i < B; ++i) {
+                const int y = y0 + i * rows;
+                const int x = 2 * lx + ((y + h) & 1);
+                if (y < ny && x < nx) {
+                    const Coef<T> c = tail_coef<T>(L.coef + 4 * tail_class(y, ny) + tail_class(x, nx));
+                    const T* q = L.u + y * pu + x;
+                    v[i] = gs_update<T>(c, L.b[y * nx + x], q[-1], q[1], q[-pu], q[pu]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < B; ++i) {
+                const int y = y0 + i * rows;
+                const int x = 2 * lx + ((y + h) & 1);
+                if (y < ny && x < nx) L.u[y * pu + x] = v[i];
+            }
+        }
+        sync();
+    }
+}
+
+// C.b = sum of the child residuals / 4 (C.u is zero already: it was cleared at the start).
+template <class T, class Sync>
+__device__ __forceinline__ void tail_restrict(const TailLevel<T>& L, const TailLevel<T>& C, int tid, int threads,
+                                              Sync sync) {
+    const int nx = L.nx, ny = L.ny, pu = nx + 2;
+    const int sh = tail_shift(C.nx, threads);
+    const int lx = tid & ((1 << sh) - 1), ly = tid >> sh, rows = threads >> sh;
+    if (lx < C.nx)
+        for (int J = ly; J < C.ny; J += rows) {
+            T sum = T(0);
+#pragma unroll
+            for (int dy = 0; dy < 2; ++dy)
+#pragma unroll
+                for (int dx = 0; dx < 2; ++dx) {
+                    const int x = 2 * lx + dx, y = 2 * J + dy;
+                    if (x < nx && y < ny) {
+                        const Coef<T> c = tail_coef<T>(L.coef + 4 * tail_class(y, ny) + tail_class(x, nx));
+                        const T* q = L.u + y * pu + x;
+                        sum += residual_at<T>(c, L.b[y * nx + x], q[0], q[-1], q[1], q[-pu], q[pu]);
+                    }
+                }
+            C.b[J * C.nx + lx] = sum * T(0.25);
+        }
+    sync();
+}
+
+// L.u += interpolated C.u.
+template <class T, class Sync>
+__device__ __forceinline__ void tail_prolong(const TailLevel<T>& L, const TailLevel<T>& C, int tid, int threads,
+                                             Sync sync) {
+    const int nx = L.nx, ny = L.ny, pu = nx + 2, pc = C.nx + 2;
+    const int sh = tail_shift(nx, threads);
+    const int lx = tid & ((1 << sh) - 1), ly = tid >> sh, rows = threads >> sh;
+    for (int x = lx; x < nx; x += 1 << sh) {
+        const T wx = L.wx[x];
+        const int I = x >> 1, J = I + L.jx[x];
+        for (int y = ly; y < ny; y += rows) {
+            const T wy = L.wy[y];
+            const int Iy = y >> 1;
+            const T* r0 = C.u + Iy * pc;
+            const T* r1 = r0 + L.jy[y] * pc;
+            L.u[y * pu + x] += bilinear<T>(r0[I], r0[J], r1[I], r1[J], wx, wy);
+        }
+    }
+    sync();
+}
+
+// The V-cycle legs of levels q0 .. q1 - 1 (down; the last level of all is `last`) and q1 - 1 .. q0
+// (up) of the tail; view(q) is level q.
+template <class T, class View, class Sync>
+__device__ __forceinline__ void tail_down(View view, int q0, int q1, int last, int nu, int tid, int threads,
+                                          Sync sync) {
+    for (int q = q0; q < q1; ++q) {
+        tail_relax<T>(view(q), nu, tid, threads, sync);
+        if (q < last) tail_restrict<T>(view(q), view(q + 1), tid, threads, sync);
+    }
+}
+template <class T, class View, class Sync>
+__device__ __forceinline__ void tail_up(View view, int q0, int q1, int nu, int tid, int threads, Sync sync) {
+    for (int q = q1 - 1; q >= q0; --q) {
+        tail_prolong<T>(view(q), view(q + 1), tid, threads, sync);
+        tail_relax<T>(view(q), nu, tid, threads, sync);
+    }
+}
+
+template <class T>
+__global__ void __launch_bounds__(kTailThreads) k_tail(TailArgs<T> a) {
     extern __shared__ __align__(16) unsigned char tail_smem[];
+    __shared__ TailCoef<T> coef[kTailMaxLevels][16];
+    __shared__ TailOffsets sl[kTailMaxLevels];
+    __shared__ T wtab[2][4 * kTailMax];            // per axis, the levels one after another
+    __shared__ signed char jtab[2][4 * kTailMax];
     const int j = blockIdx.x;
     if (a.active && !a.active[j]) return;
-    const LSlice<T>* lv = a.table + a.level_off[j];
+    const int tid = threadIdx.x;
     const int kc = a.kc[j];
-    const int K = a.nlev[j] - 1;
-    if (K - kc + 1 > kTailMaxLevels) return;  // never: a 64 x 64 level has 7 levels below it
-    // shared-memory copies of levels kc .. K: u then b, dense rows; their descriptors once per CTA
-    __shared__ LSlice<T> sl[kTailMaxLevels];
-    if (threadIdx.x == 0) {
-        T* q = reinterpret_cast<T*>(tail_smem);
-        for (int k = kc; k <= K; ++k) {
-            LSlice<T> L = lv[k];
-            L.pitch = L.nx;
-            L.u = q;
-            q += (size_t)L.nx * L.ny;
-            L.b = q;
-            q += (size_t)L.nx * L.ny;
-            sl[k - kc] = L;
+    const LSlice<T>* lv = a.table + a.level_off[j];
+    const int nl = a.nlev[j] - kc;  // levels of the tail
+    if (nl > kTailMaxLevels || nl < 1) return;  // never: a 64 x 64 level has 6 levels below it
+    const LSlice<T> G = lv[kc];
+    const int n0x = G.n0x, n0y = G.n0y;
+    // shared-memory layout: the bordered iterates of all levels, then their right-hand sides
+    T* const base = reinterpret_cast<T*>(tail_smem);
+    int ucells = 0;
+    for (int q = 0; q < nl; ++q) ucells += (level_size(n0x, kc + q) + 2) * (level_size(n0y, kc + q) + 2);
+    for (int p = tid; p < ucells; p += kTailThreads) base[p] = T(0);
+    if (tid < nl) {
+        TailOffsets L{0, ucells, 0, 0, 0, 0};
+        for (int q = 0;; ++q) {
+            L.nx = level_size(n0x, kc + q);
+            L.ny = level_size(n0y, kc + q);
+            if (q == tid) break;
+            L.u += (L.nx + 2) * (L.ny + 2);
+            L.b += L.nx * L.ny;
+            L.x += L.nx;
+            L.y += L.ny;
         }
-        for (int k = kc; k < K; ++k) {
-            sl[k - kc].uc = sl[k + 1 - kc].u;
-            sl[k - kc].bc = sl[k + 1 - kc].b;
-            sl[k - kc].pitchc = sl[k + 1 - kc].pitch;
-        }
+        sl[tid] = L;
+    }
+    auto view = [&](int q) {
+        const TailOffsets o = sl[q];
+        TailLevel<T> L;
+        L.u = base + o.u + (o.nx + 2) + 1;
+        L.b = base + o.b;
+        L.coef = coef[q];
+        L.wx = wtab[0] + o.x;
+        L.wy = wtab[1] + o.y;
+        L.jx = jtab[0] + o.x;
+        L.jy = jtab[1] + o.y;
+        L.nx = o.nx;
+        L.ny = o.ny;
+        return L;
+    };
+    for (int p = tid; p < nl * 16; p += kTailThreads) {
+        const int k = kc + (p >> 4), nx = level_size(n0x, k), ny = level_size(n0y, k);
+        auto rep = [](int cls, int n) { return cls == 0 ? 0 : (cls == 1 ? min(1, n - 1) : max(0, n - 4 + cls)); };
+        const int x = rep(p & 3, nx), y = rep((p >> 2) & 3, ny);
+        const Coef<T> c = coef_at<T>(x, y, nx, ny, n0x, n0y, k, a.alpha, T(ldexp(1.0, -2 * k)));
+        TailCoef<T>& t = coef[p >> 4][p & 15];
+        t.cw = c.cw; t.ce = c.ce; t.cn = c.cn; t.cs = c.cs; t.iD = c.iD; t.D = c.D;
     }
     __syncthreads();
-    {   // level kc from global memory: its rhs, and its iterate when continuing at level 0
-        const LSlice<T>& G = lv[kc];
-        const LSlice<T>& L = sl[0];
-        const bool cont = a.cont && kc == 0;
-        for (int p = threadIdx.x; p < L.nx * L.ny; p += blockDim.x) {
-            const int y = p / L.nx, x = p - y * L.nx;
-            const int64_t g = (int64_t)y * G.pitch + x;
-            L.b[p] = G.b[g];
-            L.u[p] = cont ? G.u[g] : T(0);  // coarse levels solve for a correction from zero
-        }
-        __syncthreads();
-    }
-    for (int k = kc; k <= K; ++k) {
-        const LSlice<T>& L = sl[k - kc];
-        const T sk = T(ldexp(1.0, -2 * k));
-        if (k > kc) {
-            for (int p = threadIdx.x; p < L.nx * L.ny; p += blockDim.x) L.u[p] = T(0);
-            __syncthreads();
-        }
-        tail_relax<T>(L, k, a.alpha, sk, a.nu_pre);
-        if (k < K) {
-            const LSlice<T>& C = sl[k + 1 - kc];
-            for (int p = threadIdx.x; p < C.nx * C.ny; p += blockDim.x) {
-                const int J = p / C.nx, I = p - J * C.nx;
-                T sum = T(0);
-#pragma unroll
-                for (int dy = 0; dy < 2; ++dy)
-#pragma unroll
-                    for (int dx = 0; dx < 2; ++dx) {
-                        const int x = 2 * I + dx, y = 2 * J + dy;
-                        if (x < L.nx && y < L.ny) {
-                            const Coef<T> c = coef_at<T>(x, y, L.nx, L.ny, L.n0x, L.n0y, k, a.alpha, sk);
-                            const int64_t q = (int64_t)y * L.pitch + x;
-                            const T uw = x > 0 ? L.u[q - 1] : T(0);
-                            const T ue = x + 1 < L.nx ? L.u[q + 1] : T(0);
-                            const T un = y > 0 ? L.u[q - L.pitch] : T(0);
-                            const T us = y + 1 < L.ny ? L.u[q + L.pitch] : T(0);
-                            sum += residual_at<T>(c, L.b[q], L.u[q], uw, ue, un, us);
-                        }
-                    }
-                C.b[(int64_t)J * C.pitch + I] = sum * T(0.25);
+    {   // interpolation tables (every level but the last), and level kc from global memory: its
+        // rhs, and its iterate when continuing at level 0
+        for (int q = 0; q + 1 < nl; ++q)
+            for (int p = tid; p < sl[q].nx + sl[q].ny; p += kTailThreads) {
+                const bool ax = p < sl[q].nx;
+                const int i = ax ? p : p - sl[q].nx;
+                int I, J;
+                T w;
+                interp_axis<T>(i, ax ? n0x : n0y, kc + q, ax ? sl[q + 1].nx : sl[q + 1].ny, I, J, w);
+                const int at = (ax ? sl[q].x : sl[q].y) + i;
+                wtab[ax ? 0 : 1][at] = w;
+                jtab[ax ? 0 : 1][at] = (signed char)(J - I);
             }
-            __syncthreads();
-        }
+        const TailLevel<T> L = view(0);
+        const bool cont = a.cont && kc == 0;
+        const int sh = tail_shift(L.nx, kTailThreads);
+        for (int x = tid & ((1 << sh) - 1); x < L.nx; x += 1 << sh)
+            for (int y = tid >> sh; y < L.ny; y += kTailThreads >> sh) {
+                const int64_t g = (int64_t)y * G.pitch + x;
+                L.b[y * L.nx + x] = G.b[g];
+                if (cont) L.u[y * (L.nx + 2) + x] = G.u[g];  // else zero: coarse levels solve for a correction
+            }
     }
-    for (int k = K - 1; k >= kc; --k) {
-        const LSlice<T>& L = sl[k - kc];
-        const T sk = T(ldexp(1.0, -2 * k));
-        for (int p = threadIdx.x; p < L.nx * L.ny; p += blockDim.x) {
-            const int y = p / L.nx, x = p - y * L.nx;
-            L.u[(int64_t)y * L.pitch + x] += prolong_at<T>(L.uc, L.pitchc, x, y, L.ncx, L.ncy, L.n0x, L.n0y, k);
-        }
-        __syncthreads();
-        tail_relax<T>(L, k, a.alpha, sk, a.nu_post);
+    __syncthreads();
+    int qs = 0;  // first level that one warp runs alone (the last level is 1 x 1)
+    while (sl[qs].nx > 8 || sl[qs].ny > 8) ++qs;
+    auto block_sync = [] { __syncthreads(); };
+    auto warp_sync = [] { __syncwarp(); };
+    tail_down<T>(view, 0, qs, nl - 1, a.nu_pre, tid, kTailThreads, block_sync);
+    if (tid < 32) {
+        tail_down<T>(view, qs, nl, nl - 1, a.nu_pre, tid, 32, warp_sync);
+        tail_up<T>(view, qs, nl - 1, a.nu_post, tid, 32, warp_sync);
     }
+    __syncthreads();
+    tail_up<T>(view, 0, qs, a.nu_post, tid, kTailThreads, block_sync);
     {   // the final iterate of level kc back to global memory
-        const LSlice<T>& G = lv[kc];
-        const LSlice<T>& L = sl[0];
-        for (int p = threadIdx.x; p < L.nx * L.ny; p += blockDim.x) {
-            const int y = p / L.nx, x = p - y * L.nx;
-            G.u[(int64_t)y * G.pitch + x] = L.u[p];
-        }
+        const TailLevel<T> L = view(0);
+        const int sh = tail_shift(L.nx, kTailThreads);
+        for (int x = tid & ((1 << sh) - 1); x < L.nx; x += 1 << sh)
+            for (int y = tid >> sh; y < L.ny; y += kTailThreads >> sh)
+                G.u[(int64_t)y * G.pitch + x] = L.u[y * (L.nx + 2) + x];
     }
 }
 

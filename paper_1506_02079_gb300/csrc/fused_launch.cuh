@@ -104,7 +104,7 @@ int launch_tail_impl(const TailArgs<T>& a, cudaStream_t st, double bytes) {
         }
     }
     KernelScope ks("coarse_tail", st, bytes);
-    fused_detail::k_tail<T><<<(unsigned)a.nslices, 512, (size_t)a.smem_bytes, st>>>(a);
+    fused_detail::k_tail<T><<<(unsigned)a.nslices, fused_detail::kTailThreads, (size_t)a.smem_bytes, st>>>(a);
     EMF_CHECK_LAUNCH();
     return EMFUSE_OK;
 }

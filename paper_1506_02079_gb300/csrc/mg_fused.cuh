@@ -216,16 +216,16 @@ __device__ __forceinline__ int find_item(const int64_t* __restrict__ ts, int n, 
 }
 
 // Shared-memory bytes of the coarse tail of a slice whose first tail level has nx x ny cells
-// (u and b of every level down to 1 x 1, dense rows).
+// (u with a border of one cell, and b, of every level down to 1 x 1).
 template <class T>
 __host__ __device__ inline size_t tail_smem_bytes(int nx, int ny) {
     size_t cells = 0;
     for (int k = 0;; ++k) {
         const int lx = ((nx - 1) >> k) + 1, ly = ((ny - 1) >> k) + 1;
-        cells += (size_t)lx * ly;
+        cells += (size_t)lx * ly + (size_t)(lx + 2) * (ly + 2);
         if (lx == 1 && ly == 1) break;
     }
-    return 2 * cells * sizeof(T);
+    return cells * sizeof(T);
 }
 
 // ---------------------------------------------------------------- fused schedule (fused.cu)
