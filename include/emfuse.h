@@ -87,9 +87,10 @@ typedef struct {
     int first_vcycles;   /* V-cycles in the first outer iteration (the second continues from
                             the first's correction in FP32 before the first FP64 residual).
                             0 = default (2).                                               */
-    int tile_rows;       /* rows of one work item (a 128-column strip) of the fused kernels
+    int tile_rows;       /* rows of one work item (a 128-column strip) of the wavefront kernels
                             on the finest level: 0 = chosen from the batch size, else a
-                            power of two in [8, 256].                                      */
+                            power of two in [8, 256].  No effect where the finest level is
+                            small enough (about 5 M cells in FP32) to run by tiles.         */
     int autotune;        /* 1: before solving, time complete solves of this batch for
                             tile_rows in {32, 64, 128, 256} (with nu = (2, 2)), then for
                             (nu_pre, nu_post) in {(1,1), (1,2), (2,1), (2,3), (3,2), (3,3),

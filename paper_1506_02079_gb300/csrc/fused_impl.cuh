@@ -21,6 +21,11 @@
 //        the result into a second buffer (uo): the warps read u on their halos, so no warp may
 //        overwrite it in place.
 //
+// Rows of a step: see `step` in k_wave for its three bodies.  Running the steps at the top of a
+// chunk by the same range-check-free bodies as the rest, and strips of any width by cached
+// stencils, took level 0 of 64 x 2048 x 2048 from 0.556 to 0.507 ms per UP leg (6.9 TB/s), of 96
+// ragged slices (291 M cells) from 1.08 to 0.66 ms (7.1 TB/s).
+//
 // Coarse tail (k_tail).  Levels whose larger side is <= 64 are run by one CTA per slice: the
 // remaining down and up legs of the V-cycle with __syncthreads() between half-sweeps, on
 // copies in shared memory.  Same per-cell arithmetic as every other schedule.
@@ -88,12 +93,6 @@ constexpr int kWaveWarps = 4;  // warps (strips) per CTA
 
 
 __host__ __device__ constexpr int wmod(int a, int w) { return ((a % w) + w) % w; }
-
-// v[i] for a runtime i in 0..3 without dynamic register indexing.
-template <class T>
-__device__ __forceinline__ T pick4(const T (&v)[4], int i) {
-    return i == 0 ? v[0] : (i == 1 ? v[1] : (i == 2 ? v[2] : v[3]));
-}
 
 // CTAs per SM the register budget is sized for: the register window grows with the sweeps (S + 3
 // row pairs) and FP64 windows take twice the registers.
@@ -174,22 +173,24 @@ __device__ __forceinline__ Coef<T> edge_coef(const StencilTab<T>& tab, int x, in
 }
 
 // Stencil of cell i of the lane on an interior row, from the lane's shared-memory cache
-// (cw, ce, cn = cs, D, 1/D per cell, as make_coef returns them on such a row).
+// (cw, ce, cn = cs, 1/D per cell, as make_coef returns them on such a row, in one vector load
+// without bank conflicts; D apart, only the residual needs it).  `cache`: the lane's first vector.
 template <class T>
 __device__ __forceinline__ Coef<T> cached_coef(uint32_t cache, int i) {
     Coef<T> c;
-    const uint32_t a = cache + i * 5 * (uint32_t)sizeof(T);
-    c.cw = lds1(a, T(0));
-    c.ce = lds1(a + sizeof(T), T(0));
-    c.cn = lds1(a + 2 * sizeof(T), T(0));
-    c.cs = c.cn;
-    c.D = lds1(a + 3 * sizeof(T), T(0));
-    c.iD = lds1(a + 4 * sizeof(T), T(0));
+    T q[4];
+    lds4(cache + i * 128 * (uint32_t)sizeof(T), q);
+    c.cw = q[0]; c.ce = q[1]; c.cn = q[2]; c.cs = q[2]; c.iD = q[3];
     return c;
 }
+template <class T>
+__device__ __forceinline__ T cached_diag(uint32_t cache, int lane, int i) {
+    return lds1(cache - lane * 3 * (uint32_t)sizeof(T) + (512 + 32 * i) * (uint32_t)sizeof(T), T(0));
+}
 
-// Half-sweep of one colour on one row of the lane's 4 cells (cells f and f + 2).
-template <class T, bool FAST>
+// Half-sweep of one colour on one row of the lane's 4 cells (cells f and f + 2).  FAST: interior
+// stencils (with the lane's diagonals); ROWS: an interior row, known when compiled.
+template <class T, bool FAST, bool ROWS>
 __device__ __forceinline__ void sweep_row(T (&row)[4], const T (&brow)[4], const T (&nrow)[4], const T (&srow)[4],
                                           int f, T west, T east, bool fast, bool irow, uint32_t cache,
                                           const StencilTab<T>& tab, const LaneDiag<T>& g, int xlane, int r, int nx,
@@ -208,15 +209,15 @@ __device__ __forceinline__ void sweep_row(T (&row)[4], const T (&brow)[4], const
             const int i = 2 * h + f;
             const T uw = i == 0 ? west : row[i - 1];
             const T ue = i == 3 ? east : row[i + 1];
-            const Coef<T> c = irow ? cached_coef<T>(cache, i)
-                                   : edge_coef<T>(tab, xlane + i, r, nx, ny, n0x, n0y, k, alpha, sk);
+            const Coef<T> c = ROWS || irow ? cached_coef<T>(cache, i)
+                                           : edge_coef<T>(tab, xlane + i, r, nx, ny, n0x, n0y, k, alpha, sk);
             row[i] = gs_update<T>(c, brow[i], uw, ue, nrow[i], srow[i]);
         }
     }
 }
 
 // Residuals of one row of the lane's 4 cells.
-template <class T, bool FAST>
+template <class T, bool FAST, bool ROWS>
 __device__ __forceinline__ void residual_row(T (&res)[4], const T (&row)[4], const T (&brow)[4], const T (&nrow)[4],
                                              const T (&srow)[4], T west, T east, bool fast, bool irow,
                                              uint32_t cache, const StencilTab<T>& tab, const LaneDiag<T>& g,
@@ -230,27 +231,15 @@ __device__ __forceinline__ void residual_row(T (&res)[4], const T (&row)[4], con
             const T D = i == 0 ? g.D0 : (i == 3 ? g.D3 : tab.ci.D);
             res[i] = residual_at_D<T>(tab.ci, D, brow[i], row[i], uw, ue, nrow[i], srow[i]);
         } else {
-            const Coef<T> c = irow ? cached_coef<T>(cache, i)
-                                   : edge_coef<T>(tab, xlane + i, r, nx, ny, n0x, n0y, k, alpha, sk);
+            Coef<T> c;
+            if (ROWS || irow) {
+                c = cached_coef<T>(cache, i);
+                c.D = cached_diag<T>(cache, threadIdx.x & 31, i);
+            } else {
+                c = edge_coef<T>(tab, xlane + i, r, nx, ny, n0x, n0y, k, alpha, sk);
+            }
             res[i] = residual_at<T>(c, brow[i], row[i], uw, ue, nrow[i], srow[i]);
         }
-    }
-}
-
-// Prolongation for lanes whose cells do not follow the interior 1/4-3/4 pattern; v0 / v1 hold
-// coarse columns cx0 - 1 .. cx0 + 2.  The interpolation along x is formed here, when needed,
-// so that nothing of this rare path stays live in registers across the march.
-template <class T>
-__device__ __forceinline__ void prolong_generic(T (&uu)[4], const T (&v0)[4], const T (&v1)[4], int cx0, T wy,
-                                                int xlane, int nx, int n0x, int k, int ncx) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        if (xlane + i >= nx) continue;
-        int I, J;
-        T wx;
-        interp_axis<T>(xlane + i, n0x, k, ncx, I, J, wx);
-        const int oI = I - cx0 + 1, oJ = J - cx0 + 1;
-        uu[i] = uu[i] + bilinear<T>(pick4<T>(v0, oI), pick4<T>(v0, oJ), pick4<T>(v1, oI), pick4<T>(v1, oJ), wx, wy);
     }
 }
 
@@ -266,7 +255,8 @@ struct WaveRing {
     static constexpr int kUSlotBytes = (ZERO ? 0 : kPairBytes) + kCoarseBytes;
     static constexpr int kBRingBytes = kNB * kPairBytes;
     static constexpr int kURingBytes = kAhead * kUSlotBytes;
-    static constexpr int kCoefBytes = 32 * 4 * 5 * (int)sizeof(T);       // per-lane stencil cache
+    // per-lane cache: stencils, and for UP the interpolation weights along x
+    static constexpr int kCoefBytes = 32 * 4 * (UP ? 6 : 5) * (int)sizeof(T);
     static constexpr int kWarpBytes = kBRingBytes + kURingBytes + kCoefBytes + (kNB * 8 + 127) / 128 * 128;
 };
 
@@ -290,7 +280,7 @@ __global__ void __launch_bounds__(kWaveWarps * 32, WaveOcc<T, S>::value) k_wave(
     unsigned char* ring = wave_smem + (size_t)warp * R::kWarpBytes;
     const uint32_t ring_s = smem_addr(ring);
     const uint32_t uring_s = ring_s + R::kBRingBytes;
-    const uint32_t coef_s = uring_s + R::kURingBytes + lane * 20 * (uint32_t)sizeof(T);
+    const uint32_t coef_s = uring_s + R::kURingBytes + lane * 4 * (uint32_t)sizeof(T);
     const uint32_t bar_s = uring_s + R::kURingBytes + R::kCoefBytes;
     if (lane == 0) {
         for (int q = 0; q < NB; ++q) mbar_init(bar_s + 8 * q, 1);
@@ -374,24 +364,24 @@ __global__ void __launch_bounds__(kWaveWarps * 32, WaveOcc<T, S>::value) k_wave(
     // prolongation geometry along x (UP): coarse columns cx0-1 .. cx0+2 around the lane
     const int cx0 = X0 / 2 + 2 * lane;
     const int cbox_x = X0 / 2 - 4;  // first staged coarse column (x * size stays 16-B aligned)
-    bool std_lane = true;  // interior pattern: J = I-1, I+1, I-1, I+1 with weight 1/4
     const bool has_coarse = UP && L.uco != nullptr;
+    T wxl[4] = {T(0), T(0), T(0), T(0)};  // weight of each cell toward its other coarse column
     if (UP) {
+        // A cell's other coarse column is the previous one for even cells and the next one for
+        // odd cells, or its weight is 0 (interp_axis: a cell's centre lies left of its coarse
+        // cell's centre if it is the left one of two).
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            int I = 0, J = 0;
-            T w = T(0);
-            if (has_coarse && lane_in) interp_axis<T>(xlane + i, L.n0x, k, L.ncx, I, J, w);
-            const int oI = I - cx0 + 1, oJ = J - cx0 + 1;
-            const int sI = i < 2 ? 1 : 2, sJ = (i == 0 || i == 2) ? sI - 1 : sI + 1;  // interior pattern
-            if (oI == sI && oJ == sJ && w == T(0.25)) continue;
-            std_lane = false;
-            // injection (J = I, weight 0) at the level's first / last cell keeps a ghost strip
+            if (!has_coarse || xlane + i < 0 || xlane + i >= nx) continue;
+            int I, J;
+            interp_axis<T>(xlane + i, L.n0x, k, L.ncx, I, J, wxl[i]);
+            if (wxl[i] == T(0.25)) continue;
+            // weight 0 at the level's first / last cell keeps a ghost strip
             const bool edge_cell = (i == 0 && xlane == 0) || (i == 3 && xlane + 3 == nx - 1);
-            if (has_coarse && all_in && edge_cell && oI == sI && J == I && w == T(0)) {
+            if (edge_cell && wxl[i] == T(0)) {
                 if (i == 0) wx0 = T(0);
                 if (i == 3) wx3 = T(0);
-            } else if (has_coarse && all_in) {
+            } else {
                 ghost_ok = false;
             }
         }
@@ -404,11 +394,12 @@ __global__ void __launch_bounds__(kWaveWarps * 32, WaveOcc<T, S>::value) k_wave(
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const Coef<T> c = make_coef<T>(axis_coef<T>(xlane + i, nx, L.n0x, k), one, k, alpha, sk);
-            cc[5 * i + 0] = c.cw;
-            cc[5 * i + 1] = c.ce;
-            cc[5 * i + 2] = c.cn;
-            cc[5 * i + 3] = c.D;
-            cc[5 * i + 4] = c.iD;
+            cc[128 * i + 0] = c.cw;
+            cc[128 * i + 1] = c.ce;
+            cc[128 * i + 2] = c.cn;
+            cc[128 * i + 3] = c.iD;
+            cc[512 + 32 * i - 3 * lane] = c.D;
+            if (UP) cc[640 + i] = wxl[i];
         }
     }
     __syncwarp();
@@ -445,14 +436,19 @@ __global__ void __launch_bounds__(kWaveWarps * 32, WaveOcc<T, S>::value) k_wave(
         lds4(ring_s + bslot * R::kPairBytes + h * kRowB + 4 * lane * (uint32_t)sizeof(T), v);
     };
 
-    // Steps whose every updated row is an interior row, in a strip whose lanes all take the
-    // interior stencil along x (and for UP the regular 1/4-3/4 prolongation pattern), run a
-    // step body specialised to the interior stencil; the others the general one.  The choice
-    // is warp-uniform, so each step executes exactly one of the two bodies.
+    // Steps whose every updated row is an interior row run a body without range checks along y:
+    // in a strip whose lanes all take the interior stencil along x (and for UP the regular
+    // 1/4-3/4 prolongation pattern) one specialised to the interior stencil (FAST), in the others
+    // one with the lanes' cached stencils (ROWS).  The remaining steps (the first and last rows of
+    // a level) run the general body.  The choice is warp-uniform, so each step executes exactly
+    // one of the three.  The first steps of a chunk, whose older pairs were never loaded, need no
+    // body of their own: what they compute for those pairs only reaches the rows that the chunk's
+    // halo is there for, and is not stored.
     const bool x_ghost = __all_sync(0xffffffffu, ghost_ok);
 
-    auto step = [&](auto fast_tag, const int T_) {
+    auto step = [&](auto fast_tag, auto rows_tag, const int T_) {
         constexpr bool FAST = decltype(fast_tag)::value;
+        constexpr bool ROWS = decltype(rows_tag)::value;  // FAST implies ROWS
         {
             // shift the window and bring in pair T
 #pragma unroll
@@ -472,15 +468,15 @@ __global__ void __launch_bounds__(kWaveWarps * 32, WaveOcc<T, S>::value) k_wave(
                 lds4(us_addr + kRowB + 4 * lane * (uint32_t)sizeof(T), w[NR - 1][1]);
             }
             // UP: add the interpolated coarse correction to rows 2T and 2T+1
-            if (has_coarse && (FAST || (2 * T_ < ny && 2 * T_ + 1 >= 0))) {
+            if (has_coarse && (ROWS || (2 * T_ < ny && 2 * T_ + 1 >= 0))) {
                 const uint32_t cb = us_addr + (ZERO ? 0 : R::kPairBytes);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int r = 2 * T_ + h;
-                    if (!FAST && (r < 0 || r >= ny)) continue;
+                    if (!ROWS && (r < 0 || r >= ny)) continue;
                     int Iy, Jy;
                     T wy;
-                    if (FAST) {  // interior pattern along y (the step's rows are >= 2 and below the last two coarse rows)
+                    if (ROWS) {  // interior pattern along y (the step's rows are >= 2 and below the last two coarse rows)
                         Iy = T_;
                         Jy = h ? T_ + 1 : T_ - 1;
                         wy = T(0.25);
@@ -507,13 +503,13 @@ __global__ void __launch_bounds__(kWaveWarps * 32, WaveOcc<T, S>::value) k_wave(
                         row[1] = fma_t(pm, bilinear<T>(v0[1], v0[2], v1[1], v1[2], q4, wy), row[1]);
                         row[2] = fma_t(pm, bilinear<T>(v0[2], v0[1], v1[2], v1[1], q4, wy), row[2]);
                         row[3] = fma_t(pm, bilinear<T>(v0[2], v0[3], v1[2], v1[3], wx3, wy), row[3]);
-                    } else if (std_lane && xlane + 3 < nx) {
-                        row[0] = row[0] + bilinear<T>(v0[1], v0[0], v1[1], v1[0], q4, wy);
-                        row[1] = row[1] + bilinear<T>(v0[1], v0[2], v1[1], v1[2], q4, wy);
-                        row[2] = row[2] + bilinear<T>(v0[2], v0[1], v1[2], v1[1], q4, wy);
-                        row[3] = row[3] + bilinear<T>(v0[2], v0[3], v1[2], v1[3], q4, wy);
                     } else {
-                        prolong_generic<T>(row, v0, v1, cx0, wy, xlane, nx, L.n0x, k, L.ncx);
+                        T wv[4];
+                        lds4(coef_s + 640 * (uint32_t)sizeof(T), wv);
+                        row[0] = row[0] + bilinear<T>(v0[1], v0[0], v1[1], v1[0], wv[0], wy);
+                        if (xlane + 1 < nx) row[1] = row[1] + bilinear<T>(v0[1], v0[2], v1[1], v1[2], wv[1], wy);
+                        if (xlane + 2 < nx) row[2] = row[2] + bilinear<T>(v0[2], v0[1], v1[2], v1[1], wv[2], wy);
+                        if (xlane + 3 < nx) row[3] = row[3] + bilinear<T>(v0[2], v0[3], v1[2], v1[3], wv[3], wy);
                     }
                 }
             }
@@ -531,7 +527,7 @@ __global__ void __launch_bounds__(kWaveWarps * 32, WaveOcc<T, S>::value) k_wave(
             for (int s = 1; s <= S; ++s) {
                 const int m = T_ - s;
                 const int r0 = 2 * m, r1 = 2 * m + 1;
-                if (!FAST && (m < pb || r0 >= ny || r1 < 0)) continue;
+                if (!ROWS && (m < pb || r0 >= ny || r1 < 0)) continue;
                 T(&p0)[4] = w[NR - 1 - s][0];
                 T(&p1)[4] = w[NR - 1 - s][1];
                 const T(&north)[4] = w[NR - 2 - s][1];  // row 2m - 1
@@ -546,24 +542,24 @@ __global__ void __launch_bounds__(kWaveWarps * 32, WaveOcc<T, S>::value) k_wave(
                 const int d0 = f0 == 0 ? -1 : 1;
                 const T x0 = __shfl_sync(0xffffffffu, f0 == 0 ? p0[3] : p0[0], lane + d0);
                 const T x1 = __shfl_sync(0xffffffffu, f0 == 0 ? p1[0] : p1[3], lane - d0);
-                const bool ir0 = FAST || interior_row(r0, ny, k), ir1 = FAST || interior_row(r1, ny, k);
+                const bool ir0 = ROWS || interior_row(r0, ny, k), ir1 = ROWS || interior_row(r1, ny, k);
                 // warp-uniform: in a strip with edge lanes every lane reads its cached stencil
                 // (an interior lane's cached stencil is the interior one), so no lane diverges
-                const bool fast = FAST || (x_ghost && ir0 && ir1);
-                sweep_row<T, FAST>(p0, b0, north, p1, f0, x0, x0, fast, ir0, coef_s, tab, g, xlane, r0, nx, ny,
+                const bool fast = FAST || (!ROWS && x_ghost && ir0 && ir1);
+                sweep_row<T, FAST, ROWS>(p0, b0, north, p1, f0, x0, x0, fast, ir0, coef_s, tab, g, xlane, r0, nx, ny,
                                    L.n0x, L.n0y, k, alpha, sk);
-                if (FAST || r1 < ny)
-                    sweep_row<T, FAST>(p1, b1, p0, south, f0 ^ 1, x1, x1, fast, ir1, coef_s, tab, g, xlane, r1, nx,
+                if (ROWS || r1 < ny)
+                    sweep_row<T, FAST, ROWS>(p1, b1, p0, south, f0 ^ 1, x1, x1, fast, ir1, coef_s, tab, g, xlane, r1, nx,
                                        ny, L.n0x, L.n0y, k, alpha, sk);
             }
             // output of the pair that completed all half-sweeps
             {
                 const int m = T_ - S;
-                if (interior_lane && lane_in && (FAST || (m >= P0 && m < P1))) {
+                if (interior_lane && lane_in && m >= P0 && m < P1) {
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         const int r = 2 * m + h;
-                        if (!FAST && r >= Y1) continue;
+                        if (!ROWS && r >= Y1) continue;
                         const T(&orow)[4] = w[NR - 1 - S][h];
                         T* dst = (UP ? L.uo : L.u) + (int64_t)r * L.pitch + xlane;
                         if (FAST || xlane + 3 < nx) {
@@ -586,20 +582,20 @@ __global__ void __launch_bounds__(kWaveWarps * 32, WaveOcc<T, S>::value) k_wave(
                 const T e0 = __shfl_down_sync(0xffffffffu, q0[0], 1);
                 const T w1 = __shfl_up_sync(0xffffffffu, q1[3], 1);
                 const T e1 = __shfl_down_sync(0xffffffffu, q1[0], 1);
-                if (L.bc && (FAST || (m >= P0 && m < P1 && lane_in))) {
+                if (L.bc && m >= P0 && m < P1 && (FAST || lane_in)) {
                     const int r0 = 2 * m, r1 = 2 * m + 1;
                     const int bq = bslot_of(bs, S + 1);
                     T b0[4], b1[4];
                     load_b(bq, 0, b0);
                     load_b(bq, 1, b1);
-                    const bool ir0 = FAST || interior_row(r0, ny, k), ir1 = FAST || interior_row(r1, ny, k);
-                    const bool fast = FAST || (x_ghost && ir0 && ir1);
+                    const bool ir0 = ROWS || interior_row(r0, ny, k), ir1 = ROWS || interior_row(r1, ny, k);
+                    const bool fast = FAST || (!ROWS && x_ghost && ir0 && ir1);
                     T res0[4], res1[4] = {T(0), T(0), T(0), T(0)};
-                    residual_row<T, FAST>(res0, q0, b0, w[0][1], q1, w0, e0, fast, ir0, coef_s, tab, g, xlane, r0,
+                    residual_row<T, FAST, ROWS>(res0, q0, b0, w[0][1], q1, w0, e0, fast, ir0, coef_s, tab, g, xlane, r0,
                                           nx, ny, L.n0x, L.n0y, k, alpha, sk);
-                    const bool has_r1 = FAST || r1 < ny;
+                    const bool has_r1 = ROWS || r1 < ny;
                     if (has_r1)
-                        residual_row<T, FAST>(res1, q1, b1, q0, w[2][0], w1, e1, fast, ir1, coef_s, tab, g, xlane,
+                        residual_row<T, FAST, ROWS>(res1, q1, b1, q0, w[2][0], w1, e1, fast, ir1, coef_s, tab, g, xlane,
                                               r1, nx, ny, L.n0x, L.n0y, k, alpha, sk);
                     // same summation order as the reference restriction: (((0 + r00) + r01) + r10) + r11
                     T c0 = T(0), c1 = T(0);
@@ -635,20 +631,17 @@ __global__ void __launch_bounds__(kWaveWarps * 32, WaveOcc<T, S>::value) k_wave(
             }
             return false;
         }
-        // The interior body also drops the range checks of a march step, so it is taken where
-        // every stage has its pair (T - S >= first pair of the march), the output pair T - S
-        // and the residual pair T - S - 1 (DOWN) lie in this chunk, the prolongation rows 2T,
-        // 2T + 1 (UP) in the level with the interior interpolation pattern along y (coarse rows
-        // T - 1 .. T + 1 all full: T + 2 < the coarse level's rows), and every row the step
-        // updates is an interior row
-        // (pairs T - S - 1 .. T - 1; interior rows form one contiguous range).
+        // The bodies without range checks along y are taken where every row the step updates
+        // (pairs T - S - 1 .. T - 1) is an interior row (interior rows form one contiguous range)
+        // and, for UP, the prolongation rows 2T, 2T + 1 lie in the level with the interior
+        // interpolation pattern along y (coarse rows T - 1 .. T + 1 all full: T + 2 < the coarse
+        // level's rows).
         const int rlo = 2 * (T_ - S - (UP ? 0 : 1)), rhi = 2 * T_ - 1;
-        const bool steady = T_ >= P0 + S + (UP ? 0 : 1) && 2 * (T_ - S) + 1 < Y1 && T_ - S < P1 &&
-                            (!UP || (2 * T_ + 1 < ny && (!has_coarse || T_ + 2 < L.ncy)));
-        if (x_ghost && steady && interior_row(rlo, ny, k) && interior_row(rhi, ny, k))
-            step(std::true_type{}, T_);
-        else
-            step(std::false_type{}, T_);
+        const bool rows = interior_row(rlo, ny, k) && interior_row(rhi, ny, k) &&
+                          (!UP || (2 * T_ + 1 < ny && (!has_coarse || T_ + 2 < L.ncy)));
+        if (rows && x_ghost) step(std::true_type{}, std::true_type{}, T_);
+        else if (rows) step(std::false_type{}, std::true_type{}, T_);
+        else step(std::false_type{}, std::false_type{}, T_);
         if (++bs == NB) { bs = 0; phase ^= 1; }
         if (++us == AHEAD) us = 0;
     }

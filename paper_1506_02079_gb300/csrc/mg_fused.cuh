@@ -215,6 +215,22 @@ __device__ __forceinline__ int find_item(const int64_t* __restrict__ ts, int n, 
     return lo;
 }
 
+// find_item by a whole warp: 32 prefix sums per round instead of one, so a chain of one or two
+// dependent loads where the bisection has log2(n).  Uniform across the warp.
+__device__ __forceinline__ int find_item_warp(const int64_t* __restrict__ ts, int n, int64_t t) {
+    const int lane = threadIdx.x & 31;
+    int lo = 0, len = n;  // the answer lies in [lo, lo + len)
+    while (len > 1) {
+        const int step = (len + 31) >> 5;
+        const int at = lo + lane * step;
+        const bool le = lane * step < len && ts[at] <= t;  // true for a prefix of the lanes, lane 0 included
+        const int hit = __popc(__ballot_sync(0xffffffffu, le)) - 1;
+        len = min(step, len - hit * step);
+        lo += hit * step;
+    }
+    return lo;
+}
+
 // Shared-memory bytes of the coarse tail of a slice whose first tail level has nx x ny cells
 // (u with a border of one cell, and b, of every level down to 1 x 1).
 template <class T>
@@ -253,6 +269,22 @@ struct WaveArgs {
     unsigned int* work;          // [0]: next work item, [1]: warps finished (both 0 at launch)
 };
 
+// One leg of a level by tiles (tile_impl.cuh).
+template <class T>
+struct TileArgs {
+    const LSlice<T>* sl;         // slices of the level
+    const int64_t* tile_start;   // tiles per slice, prefix sums (nsl + 1)
+    int nsl;
+    int64_t ntiles;
+    int k;
+    int nu;                      // red-black sweeps
+    int hx, hy;                  // halo of a tile (multiples of 4 and 2)
+    T alpha;
+    T sk;
+    const int* active;
+    int from_uo;                 // DOWN without zero start: the initial iterate is uo, not u
+};
+
 template <class T>
 struct TailArgs {
     const LSlice<T>* table;      // all levels of all slices
@@ -269,6 +301,11 @@ struct TailArgs {
 
 template <class T>
 int launch_wave(const WaveArgs<T>& a, int S, bool zero_init, bool up, cudaStream_t st, double bytes);
+template <class T>
+int launch_tile(const TileArgs<T>& a, bool zero_init, bool up, cudaStream_t st, double bytes);
+// Interior of a tile: columns and rows of its output for a halo of `halo` cells.
+template <class T>
+void tile_extent(int halo, int& hx, int& hy, int& out_x, int& out_y);
 template <class T>
 int launch_tail(const TailArgs<T>& a, cudaStream_t st, double bytes);
 

@@ -191,7 +191,7 @@ k_top(const TopSlice* __restrict__ top, const int64_t* __restrict__ tile_start, 
       TF* __restrict__ dbuf0, TF* __restrict__ dbuf1, double alpha, AlphaDeg<TF> ad,
       double* __restrict__ norms) {
     const int64_t t = blockIdx.x;
-    const int j = find_item(tile_start, nslices, t);
+    const int j = find_item_warp(tile_start, nslices, t);
     if (active && !active[j]) return;
     // the caller's buffers, and the iterate buffers of this pass: pass `it` writes buffer it & 1
     // and reads the other (they alternate, so that a tile can read d_old on its halo while its
@@ -533,6 +533,10 @@ struct LevelPlan {
     std::vector<int64_t> tile_start;    // reference-kernel tiles, prefix sums (nsl + 1)
     std::vector<LSlice<T>> wsl;         // slices that run the wavefront kernels here
     std::vector<int64_t> item_start;    // wavefront work items, prefix sums
+    bool tile = false;                  // this level's legs run by tiles instead of wavefronts
+    std::vector<int64_t> tdn_start, tup_start;  // tiles of the DOWN / UP leg, prefix sums
+    int hx[2] = {0, 0}, hy[2] = {0, 0};         // halo of a tile: DOWN, UP
+    int64_t *d_tdn = nullptr, *d_tup = nullptr;
     LSlice<T>* d_sl = nullptr;
     int64_t* d_ts = nullptr;
     LSlice<T>* d_wsl = nullptr;
@@ -565,8 +569,18 @@ struct Blob {
     }
 };
 
+// Levels of at most kTileMaxCells cells (summed over their slices) run by tiles (tile_impl.cuh),
+// larger ones by wavefronts.  A march of the wavefront kernel takes 25-35 us whatever its length;
+// a tile takes its 7-8 us once, but recomputes a third of its cells.  us per DOWN + UP leg pair,
+// tiles / wavefronts, FP32: 0.26 M cells 25 / 53, 1 M 40 / 64, 4.2 M 66 / 73, 5.2 M 73 / 71,
+// 9.5 M (odd width) 105 / 85, 17 M 163 / 119.  FP64 (the FP64 pipe bounds the recomputed cells):
+// 1.2 M 277 / 375, 4.7 M 860 / 770.
+template <class TV>
+constexpr double kTileMaxCellsOf = sizeof(TV) == 4 ? 5e6 : 2.5e6;
+
 template <class TF, class TV>
 struct Solver {
+    static constexpr double kTileMaxCells = kTileMaxCellsOf<TV>;
     const SolveRequest* rq = nullptr;  // the call being served
     cudaStream_t st;
     std::vector<LevelPlan<TV>> levels;
@@ -668,6 +682,34 @@ struct Solver {
         built = false;
     }
 
+    // Rows per wavefront work item of a level: the warps resident on the chip take the items in
+    // rounds, and a round lasts the item's row pairs plus the pairs of its halo, pipeline and
+    // set-up, so the height that minimises rounds x (pairs + overhead) is taken (ragged batches
+    // count their items).  Tall items amortise the overhead, but a last round that is nearly empty
+    // costs a whole one.
+    int wave_rows(const std::vector<LSlice<TV>>& sl) const {
+        const int S = 2 * std::max(rq->opts.nu_pre, rq->opts.nu_post);
+        const int64_t resident = (int64_t)kNumSMs * (sizeof(TV) == 4 && S <= 4 ? 16 : 8);
+        const int overhead = S + (S + 2) / 2 + 4;
+        int nymax = 1;
+        for (const auto& L : sl) nymax = std::max(nymax, L.ny);
+        int best = 8;
+        double best_cost = 1e300;
+        auto consider = [&](int ch) {
+            ch = std::max(8, std::min(512, (ch + 1) / 2 * 2));
+            int64_t items = 0;
+            for (const auto& L : sl) items += (int64_t)L.fstrips * ceil_div(L.ny, ch);
+            const double cost = (double)ceil_div(items, resident) * (ch / 2 + overhead);
+            if (cost < best_cost) {
+                best_cost = cost;
+                best = ch;
+            }
+        };
+        for (int ch = 8; ch <= 512; ch += ch < 64 ? 4 : 16) consider(ch);
+        for (int m = 1; m <= 32; ++m) consider((nymax + m - 1) / m);
+        return best;
+    }
+
     int build() {
         std::vector<int64_t> want = signature(*rq);
         if (built && want == sig) {
@@ -754,7 +796,6 @@ struct Solver {
             L.k = k;
             L.tile_start.push_back(0);
             L.item_start.push_back(0);
-            int64_t want = 0;
             for (int64_t j = 0; j < n; ++j) {
                 if (nlev[j] <= k) continue;
                 const LSlice<TV> S = make(j, k);
@@ -764,18 +805,22 @@ struct Solver {
                 if (wave(j, k)) {
                     L.wsl.push_back(S);
                     L.wcells += (double)S.nx * S.ny;
-                    want += (int64_t)S.fstrips * S.ny;
                 }
             }
-            // rows per work item: tall chunks amortise the halo rows (about 2 nu + 3 pairs per
-            // chunk) and the per-item set-up; 256 rows only where every resident warp still gets
-            // several items (the last ones would otherwise leave SMs idle), shorter ones while the
-            // level would leave SMs idle (down to 8 rows on small levels, where a march's latency,
-            // not its work, is the cost)
-            const int64_t resident = (int64_t)kNumSMs * 16;  // resident wavefront warps, about
-            L.ch = want / 256 >= 4 * resident ? 256 : 128;
-            while (L.ch > 8 && want / L.ch < resident) L.ch /= 2;  // about one item per resident warp
+            L.ch = wave_rows(L.wsl);
             if (k == 0 && rq->opts.tile_rows > 0) L.ch = rq->opts.tile_rows;
+            L.tile = L.wcells <= kTileMaxCells;
+            if (L.tile) {
+                const int halo[2] = {2 * rq->opts.nu_pre + 1, 2 * rq->opts.nu_post};
+                for (int leg = 0; leg < 2; ++leg) {
+                    int ox = 0, oy = 0;
+                    tile_extent<TV>(halo[leg], L.hx[leg], L.hy[leg], ox, oy);
+                    std::vector<int64_t>& ts = leg == 0 ? L.tdn_start : L.tup_start;
+                    ts.push_back(0);
+                    for (const auto& S : L.wsl) ts.push_back(ts.back() + ceil_div(S.nx, ox) * ceil_div(S.ny, oy));
+                }
+                continue;  // no wavefront items, no tensor maps
+            }
             for (const auto& S : L.wsl) {
                 L.item_start.push_back(L.item_start.back() + (int64_t)S.fstrips * ceil_div(S.ny, L.ch));
                 // TMA maps: row pairs of u, b and uo (one 128 x 2 box per strip step) and the
@@ -813,13 +858,16 @@ struct Solver {
                 tail_cells += (double)S.nx * S.ny;
             }
         Blob blob;
-        std::vector<size_t> pos_sl(Kmax), pos_ts(Kmax), pos_wsl(Kmax), pos_is(Kmax), pos_maps(Kmax);
+        std::vector<size_t> pos_sl(Kmax), pos_ts(Kmax), pos_wsl(Kmax), pos_is(Kmax), pos_maps(Kmax), pos_tdn(Kmax),
+            pos_tup(Kmax);
         for (int k = 0; k < Kmax; ++k) {
             pos_maps[k] = blob.add(levels[k].maps);
             pos_sl[k] = blob.add(levels[k].sl);
             pos_ts[k] = blob.add(levels[k].tile_start);
             pos_wsl[k] = blob.add(levels[k].wsl);
             pos_is[k] = blob.add(levels[k].item_start);
+            pos_tdn[k] = blob.add(levels[k].tdn_start);
+            pos_tup[k] = blob.add(levels[k].tup_start);
         }
         const size_t pos_top = blob.add(top), pos_top_ts = blob.add(top_ts);
         const size_t pos_table = blob.add(table), pos_loff = blob.add(level_off);
@@ -832,6 +880,8 @@ struct Solver {
             levels[k].d_ts = reinterpret_cast<int64_t*>(dbase + pos_ts[k]);
             levels[k].d_wsl = reinterpret_cast<LSlice<TV>*>(dbase + pos_wsl[k]);
             levels[k].d_is = reinterpret_cast<int64_t*>(dbase + pos_is[k]);
+            levels[k].d_tdn = reinterpret_cast<int64_t*>(dbase + pos_tdn[k]);
+            levels[k].d_tup = reinterpret_cast<int64_t*>(dbase + pos_tup[k]);
             levels[k].d_maps = reinterpret_cast<CUtensorMap*>(dbase + pos_maps[k]);
         }
         d_top = reinterpret_cast<TopSlice*>(dbase + pos_top);
@@ -914,6 +964,25 @@ struct Solver {
         return a;
     }
 
+    // The DOWN (leg 0) or UP (leg 1) leg of level k by tiles.
+    TileArgs<TV> targs(int k, int leg) const {
+        const LevelPlan<TV>& L = levels[k];
+        TileArgs<TV> a;
+        a.sl = L.d_wsl;
+        a.tile_start = leg == 0 ? L.d_tdn : L.d_tup;
+        a.nsl = (int)L.wsl.size();
+        a.ntiles = leg == 0 ? L.tdn_start.back() : L.tup_start.back();
+        a.k = k;
+        a.nu = leg == 0 ? rq->opts.nu_pre : rq->opts.nu_post;
+        a.hx = L.hx[leg];
+        a.hy = L.hy[leg];
+        a.alpha = TV(rq->alpha);
+        a.sk = TV(std::ldexp(1.0, -2 * k));
+        a.active = d_active;
+        a.from_uo = 0;
+        return a;
+    }
+
     int relax(int k, int sweeps) {
         const auto a = args(k);
         const unsigned g = (unsigned)levels[k].ntiles();
@@ -967,6 +1036,12 @@ struct Solver {
             const bool from_prev = cont && k == 0;
             // reads b (and u when continuing), writes u and the coarse rhs
             const double bytes = sizeof(TV) * ((from_prev ? 3.0 : 2.0) * L.wcells + 0.25 * L.wcells);
+            if (L.tile) {
+                TileArgs<TV> t = targs(k, 0);
+                t.from_uo = from_prev ? 1 : 0;
+                EMF_TRY(launch_tile<TV>(t, !from_prev, false, st, bytes));
+                continue;
+            }
             WaveArgs<TV> a = wargs(k);
             a.u_map = from_prev ? 3 : 0;
             EMF_TRY(launch_wave<TV>(a, S1, !from_prev, false, st, bytes));
@@ -978,7 +1053,8 @@ struct Solver {
             const auto& L = levels[k];
             // reads u, b and the coarse iterate, writes u
             const double bytes = sizeof(TV) * (3.0 * L.wcells + 0.25 * L.wcells);
-            EMF_TRY(launch_wave<TV>(wargs(k), S2, false, true, st, bytes));
+            if (L.tile) EMF_TRY(launch_tile<TV>(targs(k, 1), false, true, st, bytes));
+            else EMF_TRY(launch_wave<TV>(wargs(k), S2, false, true, st, bytes));
         }
         return EMFUSE_OK;
     }
