@@ -241,15 +241,14 @@ int emfuse_autotune_result(emfuse_tune_entry* out, int max_entries);
  * Direct solve of Eq. (1) by fast Fourier transforms: the frequency-space form of Sec. 3
  * ("Frequency-Space Interpretation"; the FFT solver that Sec. 3 "Alternate Solutions" weighs
  * against multigrid), as an exact second solver to compare the multigrid against.  For every
- * slice, f = o + d with d = alpha A^{-1} (s - o) computed on the mirror extension of the slice
- * to 2ny x 2nx (whose periodic Laplacian is the Neumann one of the slice) by one batched
- * real-to-complex FFT, a per-frequency scaling by alpha / (alpha + lambda), and one inverse FFT
- * (cuFFT).
+ * slice, f = o + d with d = alpha A^{-1} (s - o) computed by a two-dimensional DCT-II (whose modes
+ * diagonalise the Neumann Laplacian), a per-mode scaling by alpha / (alpha + lambda), and the
+ * inverse DCT; the cosine transforms run as batched real FFTs of the slice's own size (cuFFT).
  *   s, o, f     device float32, nslices dense slices of ny x nx (uniform batch).
  *   precision   EMFUSE_PREC_FP32 or EMFUSE_PREC_FP64 (transforms and scaling in that type).
- * Temporaries: the extended slices and their spectra (about 4 and 4 times the slices, in the
- * chosen type), from the library's pool; cuFFT plans are cached per size, batch and precision
- * until emfuse_release_cache().  Asynchronous on `stream`.
+ * Temporaries: a copy of the slices and their half spectra (about 1 and 1 times the slices, in
+ * the chosen type), from the library's pool; cuFFT plans and the tables of a size are cached per
+ * size, batch and precision until emfuse_release_cache().  Asynchronous on `stream`.
  */
 int emfuse_screened_poisson_dct(const float* s, const float* o, float* f, int64_t nslices, int64_t nx,
                                 int64_t ny, double alpha, int precision, void* stream);
@@ -264,14 +263,14 @@ int emfuse_screened_poisson_dct(const float* s, const float* o, float* f, int64_
  * orthonormal DCT-II along z (a dense nz x nz matrix applied to every pixel column, cuBLAS
  * GEMM) diagonalises L_z, which splits the problem into nz slice problems
  * (alpha + lambda_z[k]) d_k + L_xy d_k = -lambda_z[k] I_k; those are solved at once by the
- * batched mirror-extension FFT of emfuse_screened_poisson_dct, and the inverse z transform
+ * batched cosine transforms of emfuse_screened_poisson_dct, and the inverse z transform
  * (GEMM) gives d.
  *   in          device, nz x ny x nx dense [z][y][x], uint8 (dt = EMFUSE_U8) or float32.
  *   out         device float32, same shape; must not alias in.
  *   alpha       > 0 (finite).
  *   precision   EMFUSE_PREC_FP32 or EMFUSE_PREC_FP64 (transforms and scaling in that type).
- * Temporaries: two copies of the stack, its mirror extension and half spectrum (about 10
- * times the stack's cells in the chosen type) plus cuFFT's work area, from the library's pool;
+ * Temporaries: two copies of the stack and its half spectrum (about 3 times the stack's cells
+ * in the chosen type), from the library's pool, plus cuFFT's work area;
  * EMFUSE_ENOMEM when they do not fit.  The cuFFT plan (per shape and precision) and the
  * cuBLAS handle are cached until emfuse_release_cache().  Asynchronous on `stream`.
  */

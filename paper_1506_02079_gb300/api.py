@@ -340,7 +340,7 @@ def emfuse_screened_poisson(s, o, alpha: float, opts: SolveOpts | None = None, *
 
 def emfuse_screened_poisson_dct(s: torch.Tensor, o: torch.Tensor, alpha: float, precision: int = PREC_FP64,
                                 out: torch.Tensor | None = None) -> torch.Tensor:
-    """Direct solve of Eq. (1) by fast transforms (cuFFT on the mirror-extended slices) for a
+    """Direct solve of Eq. (1) by fast cosine transforms (cuFFT) for a
     uniform batch: ``s``, ``o`` CUDA float32 [z][y][x] or [y][x]; precision PREC_FP32 / PREC_FP64."""
     _require_cuda(s, o)
     s3 = s[None] if s.dim() == 2 else s
@@ -358,8 +358,8 @@ def emfuse_smooth_gradient_domain(stack: torch.Tensor, alpha: float, precision: 
                                   out: torch.Tensor | None = None) -> torch.Tensor:
     """Phase 1 as the 3-D gradient-domain problem of the earlier method (Sec. 3 "Alternate
     Solutions": target gradients with their z-components zeroed, screened by alpha), solved
-    exactly: a DCT along z (GEMM) splits it into slice problems solved by the batched
-    mirror-extension FFT.  ``stack`` CUDA uint8 or float32
+    exactly: a DCT along z (GEMM) splits it into slice problems solved by batched fast
+    cosine transforms.  ``stack`` CUDA uint8 or float32
     [z][y][x]; precision PREC_FP32 / PREC_FP64.  Returns float32 of the same shape."""
     _require_cuda(stack)
     if stack.dim() != 3 or not stack.is_contiguous():
