@@ -13,22 +13,27 @@
 //   * restriction: the sum of the (up to 8) child residuals / 8; prolongation: trilinear
 //     interpolation between true cell centres; red-black Gauss-Seidel (colour = parity of
 //     x + y + z) with nu_pre / nu_post sweeps;
-//   * V-cycles in FP32 on the correction equation, outer defect-correction passes in FP64:
-//     d += e, r = -L_z I0 - A d (every operation and the norms in FP64), out = I0 + d, until
-//     ||r|| / ||alpha I0 + L_xy I0|| <= tol.
-// One thread per cell (one per cell of the updated colour in the relaxation); the level-0
-// passes are HBM bound.  The host checks the residual norm after every defect pass.
+//   * V-cycles in FP32 on the correction equation, outer defect-correction passes: d += e,
+//     r = -L_z I0 - A d, out = I0 + d, until ||r|| / ||alpha I0 + L_xy I0|| <= tol; d and A d in
+//     two floats per value (48 bits, split.cuh), in FP64 for tol < 1e-7.
+//
+// A leg of a level is one pass over memory (k3_leg: the red-black half-sweeps pipelined along z,
+// with the prolongation before or the restriction after them); levels of at most kTail3 cells
+// run in one CTA (k3_tail).  The host checks the residual norm after every defect pass.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "emfuse_common.cuh"
 #include "emfuse_internal.cuh"
 #include "fpconv.cuh"
 #include "mg_fused.cuh"
+#include "split.cuh"
 
 namespace emfuse {
 namespace {
@@ -36,33 +41,28 @@ namespace {
 constexpr int kThreads3 = 256;
 
 struct Lev3 {
-    float* u;
-    float* b;
+    float* u;       // iterate of the V-cycle
+    float* v;       // second iterate: a leg reads one and writes the other
+    float* b;       // right-hand side
     int nx, ny, nz;
-};
-
-struct AdegTab {
-    double v[7];  // alpha + q, q = 0..6 (the diagonal of A for a cell with q neighbours)
+    int pitch;      // row pitch of u and b (even); v has its own
+    int vpitch;
 };
 
 struct Geo3 {
     int n0x, n0y, n0z;  // finest sizes (fix the cell geometry of every level)
 };
 
-__device__ __forceinline__ int64_t idx3(int x, int y, int z, int nx, int ny) {
-    return ((int64_t)z * ny + y) * nx + x;
-}
-
-// The 7-point finite-volume stencil of level k at cell (x, y, z).
-struct Coef3 {
-    float cw, ce, cn, cs, cd, cu, D;
+// The 7-point finite-volume stencil of level k at a cell.
+struct alignas(16) Coef3 {
+    float cw, ce, cn, cs, cd, cu, iD, D;
 };
 
-__device__ __forceinline__ Coef3 coef3(int x, int y, int z, const Lev3& L, const Geo3& g, int k, float alpha,
+__device__ __forceinline__ Coef3 coef3(int x, int y, int z, int nx, int ny, int nz, const Geo3& g, int k, float alpha,
                                        float sk) {
-    const AxisCoef<float> ax = axis_coef<float>(x, L.nx, g.n0x, k);
-    const AxisCoef<float> ay = axis_coef<float>(y, L.ny, g.n0y, k);
-    const AxisCoef<float> az = axis_coef<float>(z, L.nz, g.n0z, k);
+    const AxisCoef<float> ax = axis_coef<float>(x, nx, g.n0x, k);
+    const AxisCoef<float> ay = axis_coef<float>(y, ny, g.n0y, k);
+    const AxisCoef<float> az = axis_coef<float>(z, nz, g.n0z, k);
     Coef3 c;
     const float ayz = ay.w * az.w, axz = ax.w * az.w, axy = ax.w * ay.w;
     c.cw = sk * (ayz * ax.gm);
@@ -72,129 +72,602 @@ __device__ __forceinline__ Coef3 coef3(int x, int y, int z, const Lev3& L, const
     c.cd = sk * (axy * az.gm);
     c.cu = sk * (axy * az.gp);
     c.D = fmaf(alpha, axy * az.w, ((c.cw + c.ce) + (c.cn + c.cs)) + (c.cd + c.cu));
+    c.iD = 1.f / c.D;
     return c;
 }
 
-// sum_q c_pq u_q over the neighbours that exist (a zero coefficient marks a missing one)
-__device__ __forceinline__ float nbr_sum(const float* __restrict__ u, const Coef3& c, int x, int y, int z,
-                                         const Lev3& L) {
-    const int64_t p = idx3(x, y, z, L.nx, L.ny);
-    const int64_t sy = L.nx, sz = (int64_t)L.nx * L.ny;
-    float acc = 0.f;
-    if (c.cw != 0.f) acc = fmaf(c.cw, u[p - 1], acc);
-    if (c.ce != 0.f) acc = fmaf(c.ce, u[p + 1], acc);
-    if (c.cn != 0.f) acc = fmaf(c.cn, u[p - sy], acc);
-    if (c.cs != 0.f) acc = fmaf(c.cs, u[p + sy], acc);
-    if (c.cd != 0.f) acc = fmaf(c.cd, u[p - sz], acc);
-    if (c.cu != 0.f) acc = fmaf(c.cu, u[p + sz], acc);
-    return acc;
+// Class of index i of an axis of n cells: 0 first, 1 inner, 2 last but one, 3 last.  axis_coef is
+// the same for all inner cells, so a level has at most 4 x 4 x 4 different stencils.
+__device__ __forceinline__ int class3(int i, int n) {
+    return i >= 1 && i + 2 < n ? 1 : (i == 0 ? 0 : (i == n - 1 ? 3 : 2));
+}
+__device__ __forceinline__ int class_rep(int c, int n) {  // a cell of class c (if the axis has one)
+    return c == 0 ? 0 : (c == 1 ? min(1, n - 1) : max(0, n - 4 + c));
+}
+// Entry t of a level's table, [class of z][class of y][class of x].
+__device__ __forceinline__ Coef3 table_entry(int t, int nx, int ny, int nz, const Geo3& g, int k, float alpha, float sk) {
+    return coef3(class_rep(t & 3, nx), class_rep((t >> 2) & 3, ny), class_rep(t >> 4, nz), nx, ny, nz, g, k, alpha, sk);
 }
 
-// Cells whose three axes are interior at level k (axis_coef gives w = 1 and both faces 1
-// there): the stencil is sk on every face and D = alpha + 6 sk.
-__device__ __forceinline__ bool interior3(int x, int y, int z, const Lev3& L, int k) {
-    return interior_row(x, L.nx, k) && interior_row(y, L.ny, k) && interior_row(z, L.nz, k);
-}
+// ---------------------------------------------------------------- one leg of a level
+// A CTA owns a tile of 64 x 64 cells in x and y (16 warps of 4 rows; a lane holds 2 cells of each
+// row) and marches along z.  At step T plane T arrives and half-sweep s (s = 1 .. S) updates plane
+// T - s: it reads the other colour of planes T - s - 1 .. T - s + 1, all of which half-sweep s - 1
+// has updated, in plane T - s + 1 earlier in this step and in plane T - s in the step before.  So
+// the S half-sweeps of a leg are one pass over memory, exactly S global half-sweeps, with one
+// barrier per plane: neighbours along z are the thread's own registers, along x in the lane or
+// one shuffle away, along y in registers or, across warps, edge rows in shared memory, written
+// in one step and read in the next.  Wrong values enter at the tile's rim (no neighbours there)
+// and move in by one cell per half-sweep: a halo of S cells (S + 1 under a residual) is
+// recomputed by the neighbouring tiles, and likewise S planes at the ends of a chunk along z.
+//
+//   DOWN  optionally from zero; after the sweeps the residual, summed 2 x 2 x 2 / 8 into the next
+//         level's right-hand side (where cb is given).
+//   UP    the interpolated coarse correction is added as a plane arrives (where cu is given); the
+//         result is stored, or added to the correction d (where d is given).
+//
+// The source and destination differ: tiles read their halo while neighbours write.
+//
+// Bound by instruction issue (about 50 per cell at S = 4, halo included) at one CTA of 16 warps
+// per SM; S = 4 keeps 7 planes in registers, the right-hand sides of the planes under way are kept
+// in shared memory.  32 x 1024 x 1024: DOWN 0.25 ms, UP with the addition to d 0.53 ms; one kernel per
+// half-sweep, restriction and prolongation took 0.89 and 0.84 (and 0.11 for the addition).
+constexpr int kWarps3 = 16, kRows3 = 4, kTile3 = 64;
 
-// The interior diagonal of level k and its reciprocal (the general formula of coef3 with unit
-// widths and faces), passed to the kernels from the host.
-struct Diag3 {
-    float D, iD;
+struct Leg3 {
+    const float* src;      // initial iterate (not read from zero)
+    float* dst;
+    const float* b;
+    float* cb;             // next level's right-hand side (DOWN) or null
+    const float* cu;       // next level's iterate (UP) or null
+    Split* d;              // UP: the correction the result is added to, instead of dst; or null
+    int sp, dp, bp, cp, pitch_d;  // row pitches
+    int svec, dvec;        // src / dst pairs are 8-byte aligned
+    int d_first;           // d = result instead of d += result
+    int nx, ny, nz, ncx, ncy, ncz;
+    int k, halo, zch;      // halo in x and y (even); planes per chunk (even)
+    unsigned tx, ty;       // tiles along x and y (block = (chunk * ty + tile row) * tx + tile column)
+    Geo3 g;
+    float alpha, sk;
 };
 
-// One red-black half-sweep: the cells of colour `colour` ((x + y + z) & 1) get
-// u = (b + sum_q c_pq u_q) / D.  One thread per pair of cells along x.
-__global__ void __launch_bounds__(kThreads3) k3_relax(Lev3 L, Geo3 g, int k, float alpha, float sk, Diag3 di,
-                                                      int colour) {
-    const int nxp = (L.nx + 1) >> 1;
-    const int64_t rows = (int64_t)L.ny * L.nz;
-    const int64_t sy = L.nx, sz = (int64_t)L.nx * L.ny;
-    for (int64_t row = blockIdx.x; row < rows; row += gridDim.x)  // one (y, z) row at a time
-    for (int xp = threadIdx.x; xp < nxp; xp += blockDim.x) {
-        const int y = int(row % L.ny), z = int(row / L.ny);
-        const int x = 2 * xp + ((y + z + colour) & 1);
-        if (x >= L.nx) continue;
-        const int64_t p = row * L.nx + x;
-        if (interior3(x, y, z, L, k)) {
-            const float* u = L.u;
-            const float acc = ((u[p - 1] + u[p + 1]) + (u[p - sy] + u[p + sy])) + (u[p - sz] + u[p + sz]);
-            L.u[p] = fmaf(sk, acc, L.b[p]) * di.iD;
-        } else {
-            const Coef3 c = coef3(x, y, z, L, g, k, alpha, sk);
-            L.u[p] = (L.b[p] + nbr_sum(L.u, c, x, y, z, L)) / c.D;
-        }
-    }
+template <int S>
+constexpr int leg3_smem() {
+    return (S + 2) * (kTile3 * kTile3 + kWarps3 * 2 * kTile3) * (int)sizeof(float);
 }
 
-// Residual of level k restricted to level k + 1: C.b = (sum of the child residuals) / 8,
-// C.u = 0.  One thread per coarse cell.
-__global__ void __launch_bounds__(kThreads3) k3_residual_restrict(Lev3 F, Lev3 C, Geo3 g, int k, float alpha,
-                                                                  float skf, Diag3 di) {
-    const int64_t rows = (int64_t)C.ny * C.nz;
-    const int64_t sy = F.nx, sz = (int64_t)F.nx * F.ny;
-    for (int64_t row = blockIdx.x; row < rows; row += gridDim.x)
-    for (int X = threadIdx.x; X < C.nx; X += blockDim.x) {
-        const int Y = int(row % C.ny), Z = int(row / C.ny);
-        const int64_t t = row * C.nx + X;
-        float sum = 0.f;
-        for (int dz = 0; dz < 2; ++dz) {
-            const int z = 2 * Z + dz;
-            if (z >= F.nz) break;
-            for (int dy = 0; dy < 2; ++dy) {
-                const int y = 2 * Y + dy;
-                if (y >= F.ny) break;
-                for (int dx = 0; dx < 2; ++dx) {
-                    const int x = 2 * X + dx;
-                    if (x >= F.nx) break;
-                    const int64_t p = idx3(x, y, z, F.nx, F.ny);
-                    if (interior3(x, y, z, F, k)) {
-                        const float* u = F.u;
-                        const float acc =
-                            ((u[p - 1] + u[p + 1]) + (u[p - sy] + u[p + sy])) + (u[p - sz] + u[p + sz]);
-                        sum += F.b[p] - fmaf(di.D, u[p], -skf * acc);
+constexpr int kOut3 = 8;  // "missing neighbours" of a column or row outside the level
+
+// Missing neighbours along one axis at index i.
+__device__ __forceinline__ int missing3(int i, int n) { return i < 0 || i >= n ? kOut3 : int(i == 0) + int(i == n - 1); }
+// All cells of an axis of n0 fine cells are full at level k.
+__device__ __forceinline__ bool full3(int n0, int k) { return (n0 & ((1 << k) - 1)) == 0; }
+
+// b + sum_q c_pq u_q by a table entry (in shared memory).
+__device__ __noinline__ float general_sum(const Coef3* q, float b, float uw, float ue, float un, float us, float ud,
+                                          float uu) {
+    float acc = fmaf(q->cw, uw, fmaf(q->ce, ue, b));
+    acc = fmaf(q->cn, un, fmaf(q->cs, us, acc));
+    return fmaf(q->cd, ud, fmaf(q->cu, uu, acc));
+}
+
+template <int S, bool ZERO, bool UP>
+__global__ void __launch_bounds__(kWarps3 * 32, 1) k3_leg(const Leg3 a) {
+    constexpr int NS = S + 2;                 // planes in the rings
+    constexpr int NP = UP ? S + 2 : S + 3;    // planes in registers: T - NP + 1 .. T
+    constexpr int R = kRows3;
+    extern __shared__ __align__(16) float smem3[];
+    float* const bring = smem3;                            // [NS][64][64] right-hand sides, own cells only
+    float* const edge = smem3 + NS * kTile3 * kTile3;      // [NS][warp][first, last row][64]
+    __shared__ Coef3 tab[64];
+    // levels of full cells: 1 / D and D of a cell with c missing neighbours, 0 for cells outside
+    __shared__ float itab[kOut3 + kOut3 + 3], dtab[kOut3 + kOut3 + 3];
+    __shared__ float roww[kTile3];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nx = a.nx, ny = a.ny, nz = a.nz, k = a.k;
+    const int ox = kTile3 - 2 * a.halo;
+    const unsigned tile = blockIdx.x / a.tx, chunk = tile / a.ty;
+    const int X0 = int(blockIdx.x - tile * a.tx) * ox, Y0 = int(tile - chunk * a.ty) * ox;  // even
+    const int x = X0 - a.halo + 2 * lane;                  // first of the lane's two columns (even)
+    const int row0 = R * warp;
+    const int y = Y0 - a.halo + row0;                      // first of the warp's rows (even)
+    const int z0 = int(chunk) * a.zch, z1 = min(z0 + a.zch, nz);
+    const int HZ = UP ? S : S + 1;
+    const int Tb = max(0, z0 - HZ);
+    const int Te = UP ? z1 - 1 + S : z1 + S;
+    if (tid < 64) tab[tid] = table_entry(tid, nx, ny, nz, a.g, k, a.alpha, a.sk);
+    if (tid < kOut3 + kOut3 + 3) {
+        const float D = a.alpha + a.sk * float(6 - min(tid, 6));
+        itab[tid] = tid < 7 ? 1.f / D : 0.f;
+        dtab[tid] = tid < 7 ? D : 0.f;
+    }
+    if (UP && tid < kTile3) {
+        const int yr = Y0 - a.halo + tid;
+        float w = 0.f;
+        if (a.cu && yr >= 0 && yr < ny) {
+            int I, J;
+            interp_axis<float>(yr, a.g.n0y, k, a.ncy, I, J, w);
+        }
+        roww[tid] = w;
+    }
+    float wx0 = 0.f, wx1 = 0.f;
+    if (UP && a.cu) {
+        int I, J;
+        if (x >= 0 && x < nx) interp_axis<float>(x, a.g.n0x, k, a.ncx, I, J, wx0);
+        if (x + 1 >= 0 && x + 1 < nx) interp_axis<float>(x + 1, a.g.n0x, k, a.ncx, I, J, wx1);
+    }
+    const bool col0 = x >= 0 && x < nx, col1 = x >= 0 && x + 1 < nx;  // x is even
+    // Where a warp's cells are all full, the stencil is the interior one with cells outside the
+    // level kept at exactly 0 (1 / D = 0): a missing neighbour adds nothing, and only the diagonal
+    // differs.  Warps and planes with partial cells (the last cell of an axis, and its neighbour)
+    // take the level's table, out of line.
+    const bool full_z = full3(a.g.n0z, k);
+    const bool full_warp = (full3(a.g.n0x, k) || X0 - a.halo + kTile3 - 1 < nx - 2) && (full3(a.g.n0y, k) || y + R - 1 < ny - 2);
+    const int mx[2] = {missing3(x, nx), missing3(x + 1, nx)};
+    unsigned my = 0;  // one nibble per row
+#pragma unroll
+    for (int r = 0; r < R; ++r) my |= (unsigned)missing3(y + r, ny) << (4 * r);
+    const bool lane_out = col0 && 2 * lane >= a.halo && 2 * lane < kTile3 - a.halo;
+    const int ylim = min(Y0 + ox, ny);
+    unsigned rows_in = 0, rows_out = 0;  // rows of the warp in the level / among the tile's output
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        rows_in |= (y + r >= 0 && y + r < ny ? 1u : 0u) << r;
+        rows_out |= (y + r >= Y0 && y + r < ylim ? 1u : 0u) << r;
+    }
+
+    float w[NP][R][2];
+#pragma unroll
+    for (int q = 0; q < NP; ++q)
+#pragma unroll
+        for (int r = 0; r < R; ++r) w[q][r][0] = w[q][r][1] = 0.f;
+    float2 pu[R], pb[R];  // plane T + 1 on its way
+    const int64_t first_row = (int64_t)Tb * ny + y;
+    const float* bsrc = a.b + first_row * a.bp + x;     // next plane to fetch, this lane's first cell
+    const float* usrc = ZERO ? nullptr : a.src + first_row * a.sp + x;
+    const int64_t bstep = (int64_t)ny * a.bp, ustep = (int64_t)ny * a.sp;
+    // (the padding of a row is masked when the plane is taken, not here, so that nothing waits for
+    // the loads before then)
+    auto fetch = [&](int z) {
+        const bool in = z < nz && col0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            pu[r] = pb[r] = make_float2(0.f, 0.f);
+            if (in && (rows_in >> r & 1)) {
+                pb[r] = *reinterpret_cast<const float2*>(bsrc + r * a.bp);
+                if (!ZERO) {
+                    const float* p = usrc + r * a.sp;
+                    if (a.svec) {
+                        pu[r] = *reinterpret_cast<const float2*>(p);
                     } else {
-                        const Coef3 c = coef3(x, y, z, F, g, k, alpha, skf);
-                        sum += F.b[p] - fmaf(c.D, F.u[p], -nbr_sum(F.u, c, x, y, z, F));
+                        pu[r].x = p[0];
+                        if (col1) pu[r].y = p[1];
                     }
                 }
             }
         }
-        C.b[t] = sum * 0.125f;
-        C.u[t] = 0.f;
-    }
-}
-
-// F.u += trilinear interpolation of C.u (level k + 1) at the fine cell centres.
-__global__ void __launch_bounds__(kThreads3) k3_prolong_add(Lev3 F, Lev3 C, Geo3 g, int k) {
-    const int64_t rows = (int64_t)F.ny * F.nz;
-    for (int64_t row = blockIdx.x; row < rows; row += gridDim.x)
-    for (int x = threadIdx.x; x < F.nx; x += blockDim.x) {
-        const int y = int(row % F.ny), z = int(row / F.ny);
-        const int64_t t = row * F.nx + x;
-        int Ix, Jx, Iy, Jy, Iz, Jz;
-        float wx, wy, wz;
-        if (x >= 2 && (x >> 1) + 2 < C.nx && y >= 2 && (y >> 1) + 2 < C.ny && z >= 2 && (z >> 1) + 2 < C.nz) {
-            // all three axes in the regular pattern of interp_axis: weight 1/4 toward the
-            // neighbouring coarse centre on the side of the fine cell
-            Ix = x >> 1; Jx = (x & 1) ? Ix + 1 : Ix - 1;
-            Iy = y >> 1; Jy = (y & 1) ? Iy + 1 : Iy - 1;
-            Iz = z >> 1; Jz = (z & 1) ? Iz + 1 : Iz - 1;
-            wx = wy = wz = 0.25f;
-        } else {
-            interp_axis<float>(x, g.n0x, k, C.nx, Ix, Jx, wx);
-            interp_axis<float>(y, g.n0y, k, C.ny, Iy, Jy, wy);
-            interp_axis<float>(z, g.n0z, k, C.nz, Iz, Jz, wz);
+        bsrc += bstep;
+        if (!ZERO) usrc += ustep;
+    };
+    fetch(Tb);
+    // UP: coarse planes zp = (T - 1) / 2 (rounded down) in h0 and zp + 1 in h1, interpolated along x at
+    // the lane's two columns, rows y/2 - 1 .. y/2 + 2; plane zp + 2 on its way (pc; pe: the column
+    // beyond the warp's edge, lanes 0 and 31).  The other coarse cell of a fine cell is the
+    // previous one for even cells and the next one for odd cells, or its weight is 0.
+    constexpr int Q = R / 2 + 2;
+    float h0[Q][2], h1[Q][2], pc[Q], pe[Q];
+    const int cx = x >> 1, cy = y >> 1;  // arithmetic shifts: y may be negative
+    const int xe = lane == 0 ? cx - 1 : cx + 1;
+    auto fetch_coarse = [&](int Z) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int Y = cy - 1 + q;
+            pc[q] = pe[q] = 0.f;
+            if (Z >= 0 && Z < a.ncz && Y >= 0 && Y < a.ncy) {
+                const float* p = a.cu + ((int64_t)Z * a.ncy + Y) * a.cp;
+                if (cx >= 0 && cx < a.ncx) pc[q] = p[cx];
+                if ((lane == 0 || lane == 31) && xe >= 0 && xe < a.ncx) pe[q] = p[xe];
+            }
         }
-        const float* u0 = C.u + (int64_t)Iz * C.ny * C.nx;
-        const float* u1 = C.u + (int64_t)Jz * C.ny * C.nx;
-        const float a = bilinear<float>(u0[(int64_t)Iy * C.nx + Ix], u0[(int64_t)Iy * C.nx + Jx],
-                                        u0[(int64_t)Jy * C.nx + Ix], u0[(int64_t)Jy * C.nx + Jx], wx, wy);
-        const float b = bilinear<float>(u1[(int64_t)Iy * C.nx + Ix], u1[(int64_t)Iy * C.nx + Jx],
-                                        u1[(int64_t)Jy * C.nx + Ix], u1[(int64_t)Jy * C.nx + Jx], wx, wy);
-        F.u[t] += fmaf(wz, b - a, a);
+    };
+    auto take_coarse = [&](float (&h)[Q][2]) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const float v = pc[q];
+            float cw = __shfl_up_sync(0xffffffffu, v, 1), ce = __shfl_down_sync(0xffffffffu, v, 1);
+            if (lane == 0) cw = pe[q];
+            if (lane == 31) ce = pe[q];
+            h[q][0] = fmaf(wx0, cw - v, v);
+            h[q][1] = fmaf(wx1, ce - v, v);
+        }
+    };
+    if (UP && a.cu) {
+        const int zp = (Tb - 1) >> 1;
+        fetch_coarse(zp);
+        take_coarse(h0);
+        fetch_coarse(zp + 1);
+        take_coarse(h1);
+        fetch_coarse(zp + 2);
+    }
+    const int64_t out_row = (int64_t)z0 * ny + y;  // next output plane, this lane's first cell
+    float* odst = a.dst + out_row * a.dp + x;
+    Split* odst_d = a.d + out_row * a.pitch_d + x;
+    const int64_t ostep = (int64_t)ny * a.dp, ostep_d = (int64_t)ny * a.pitch_d;
+    float part[2] = {0.f, 0.f};  // restriction: the even plane's 2 x 2 sums of the two coarse rows
+    int slot = Tb % NS;          // ring slot of plane T
+    auto slot_of = [&](int back) { const int q = slot - back; return q < 0 ? q + NS : q; };
+    auto edge_at = [&](int sl, int wr, int which) { return edge + ((sl * kWarps3 + wr) * 2 + which) * kTile3 + 2 * lane; };
+
+#pragma unroll 1
+    for (int T = Tb; T <= Te; ++T) {
+        __syncthreads();  // edge rows of the last step are visible, those of the oldest plane are free
+#pragma unroll
+        for (int q = 0; q + 1 < NP; ++q)
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                w[q][r][0] = w[q + 1][r][0];
+                w[q][r][1] = w[q + 1][r][1];
+            }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            w[NP - 1][r][0] = pu[r].x;
+            w[NP - 1][r][1] = col1 ? pu[r].y : 0.f;
+            if (!col1) pb[r].y = 0.f;
+            *reinterpret_cast<float2*>(bring + (slot * kTile3 + row0 + r) * kTile3 + 2 * lane) = pb[r];
+        }
+        if (T < Te) fetch(T + 1);
+        if (UP && a.cu && T < nz) {
+            if ((T & 1) && T > Tb) {  // planes (T - 1) / 2 and the next one
+#pragma unroll
+                for (int q = 0; q < Q; ++q) {
+                    h0[q][0] = h1[q][0];
+                    h0[q][1] = h1[q][1];
+                }
+                take_coarse(h1);
+                fetch_coarse(((T - 1) >> 1) + 2);
+            }
+            int Iz, Jz;
+            float wz;
+            interp_axis<float>(T, a.g.n0z, k, a.ncz, Iz, Jz, wz);
+            if ((T & 1) == 0) wz = 1.f - wz;  // weight of h1: T's own coarse plane is h1 for even T
+            float h[Q][2];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                h[q][0] = fmaf(wz, h1[q][0] - h0[q][0], h0[q][0]);
+                h[q][1] = fmaf(wz, h1[q][1] - h0[q][1], h0[q][1]);
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if (!(rows_in >> r & 1)) continue;
+                const float wy = roww[row0 + r];
+                const int q0 = r / 2 + 1, q1 = (r & 1) ? q0 + 1 : q0 - 1;
+                if (col0) w[NP - 1][r][0] += fmaf(wy, h[q1][0] - h[q0][0], h[q0][0]);
+                if (col1) w[NP - 1][r][1] += fmaf(wy, h[q1][1] - h[q0][1], h[q0][1]);
+            }
+        }
+        if (S > 0 || !UP) {
+            *reinterpret_cast<float2*>(edge_at(slot, warp, 0)) = make_float2(w[NP - 1][0][0], w[NP - 1][0][1]);
+            *reinterpret_cast<float2*>(edge_at(slot, warp, 1)) = make_float2(w[NP - 1][R - 1][0], w[NP - 1][R - 1][1]);
+        }
+        // half-sweep s of plane T - s: colour (s - 1) & 1 of x + y + z; with x and y even for cell 0 of
+        // row 0, that row's cell is I0 = (s - 1 + z) & 1 and every second row's the other
+        // (BODY 0: full cells, inner rows; 1: full cells; 2: partial cells)
+        auto half_sweep = [&](auto stage_tag, auto i_tag, auto body_tag, int m) {
+            constexpr int s = decltype(stage_tag)::value, I0 = decltype(i_tag)::value;
+            constexpr int BODY = decltype(body_tag)::value;
+            constexpr int P = NP - 1 - s;
+            const int sl = slot_of(s);
+            const float no = warp > 0 ? edge_at(sl, warp - 1, 1)[I0] : 0.f;
+            constexpr int IL = (I0 + R - 1) & 1;
+            const float so = warp + 1 < kWarps3 ? edge_at(sl, warp + 1, 0)[IL] : 0.f;
+            const int mz = int(m == 0) + int(m == nz - 1);
+            float iD[2] = {0.f, 0.f};
+            if (BODY == 0) {
+                iD[0] = itab[mx[0] + mz];
+                iD[1] = itab[mx[1] + mz];
+            }
+            const float* bp = bring + (sl * kTile3 + row0) * kTile3 + 2 * lane;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int i = (I0 + r) & 1;
+                float(&u)[2] = w[P][r];
+                const float o = i == 0 ? __shfl_up_sync(0xffffffffu, u[1], 1) : __shfl_down_sync(0xffffffffu, u[0], 1);
+                const float uw = i == 0 ? o : u[0], ue = i == 0 ? u[1] : o;
+                const float un = r > 0 ? w[P][r > 0 ? r - 1 : 0][i] : no;
+                const float us = r + 1 < R ? w[P][r + 1 < R ? r + 1 : 0][i] : so;
+                const float ud = w[P - 1][r][i], uu = w[P + 1][r][i];
+                const float bv = bp[r * kTile3 + i];
+                if (BODY < 2) {
+                    const float acc = fmaf(a.sk, ((uw + ue) + (un + us)) + (ud + uu), bv);
+                    u[i] = acc * (BODY == 0 ? iD[i] : itab[mx[i] + int(my >> (4 * r) & 15u) + mz]);
+                } else if ((i == 0 ? col0 : col1) && (rows_in >> r & 1)) {
+                    const Coef3* q = tab + class3(m, nz) * 16 + class3(y + r, ny) * 4 + class3(x + i, nx);
+                    u[i] = general_sum(q, bv, uw, ue, un, us, ud, uu) * q->iD;
+                }
+                if (r == 0) edge_at(sl, warp, 0)[i] = u[i];
+                if (r == R - 1) edge_at(sl, warp, 1)[i] = u[i];
+            }
+        };
+        auto stage = [&](auto stage_tag) {
+            constexpr int s = decltype(stage_tag)::value;
+            const int m = T - s;
+            if (m < Tb || m >= nz) return;
+            const bool full = full_warp && (full_z || m + 2 < nz);
+            auto run = [&](auto i_tag) {
+                if (full && my == 0) half_sweep(stage_tag, i_tag, std::integral_constant<int, 0>{}, m);
+                else if (full) half_sweep(stage_tag, i_tag, std::integral_constant<int, 1>{}, m);
+                else half_sweep(stage_tag, i_tag, std::integral_constant<int, 2>{}, m);
+            };
+            if (((s - 1 + m) & 1) == 0) run(std::integral_constant<int, 0>{});
+            else run(std::integral_constant<int, 1>{});
+        };
+        if constexpr (S >= 1) stage(std::integral_constant<int, 1>{});
+        if constexpr (S >= 2) stage(std::integral_constant<int, 2>{});
+        if constexpr (S >= 3) stage(std::integral_constant<int, 3>{});
+        if constexpr (S >= 4) stage(std::integral_constant<int, 4>{});
+        {   // the plane that completed all half-sweeps
+            const int m = T - S;
+            const bool mine = m >= z0 && m < z1;
+            if (mine && lane_out) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    if (!(rows_out >> r & 1)) continue;
+                    const float v0 = w[NP - 1 - S][r][0], v1 = w[NP - 1 - S][r][1];
+                    if (UP && a.d) {
+                        Split* q = odst_d + r * a.pitch_d;  // 16-byte aligned, the padding included
+                        Split e[2] = {{v0, 0.f}, {v1, 0.f}};
+                        if (!a.d_first) {
+                            const float4 t = *reinterpret_cast<const float4*>(q);
+                            e[0] = split_add(Split{t.x, t.y}, v0);
+                            e[1] = split_add(Split{t.z, t.w}, v1);
+                        }
+                        *reinterpret_cast<float4*>(q) = make_float4(e[0].hi, e[0].lo, e[1].hi, e[1].lo);
+                    } else {
+                        float* q = odst + r * a.dp;
+                        if (a.dvec) {
+                            *reinterpret_cast<float2*>(q) = make_float2(v0, v1);
+                        } else {
+                            q[0] = v0;
+                            if (col1) q[1] = v1;
+                        }
+                    }
+                }
+            }
+            if (mine) {
+                odst += ostep;
+                if (UP) odst_d += ostep_d;
+            }
+        }
+        if (!UP && a.cb) {
+            const int m = T - S - 1;
+            if (m >= z0 && m < z1) {
+                const int sl = slot_of(S + 1);
+                float2 no = make_float2(0.f, 0.f), so = no;
+                if (warp > 0) no = *reinterpret_cast<const float2*>(edge_at(sl, warp - 1, 1));
+                if (warp + 1 < kWarps3) so = *reinterpret_cast<const float2*>(edge_at(sl, warp + 1, 0));
+                const bool full = full_warp && (full_z || m + 2 < nz);
+                const int mz = int(m == 0) + int(m == nz - 1);
+                float sum[R / 2];
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    constexpr int P = UP ? 1 : NP - 2 - S;  // plane T - S - 1 (never used for UP)
+                    const float2 bv = *reinterpret_cast<const float2*>(bring + (sl * kTile3 + row0 + r) * kTile3 + 2 * lane);
+                    const float u0 = w[P][r][0], u1 = w[P][r][1];
+                    const float uw = __shfl_up_sync(0xffffffffu, u1, 1), ue = __shfl_down_sync(0xffffffffu, u0, 1);
+                    const float n0 = r > 0 ? w[P][r > 0 ? r - 1 : 0][0] : no.x, n1 = r > 0 ? w[P][r > 0 ? r - 1 : 0][1] : no.y;
+                    const float s0 = r + 1 < R ? w[P][r + 1 < R ? r + 1 : 0][0] : so.x;
+                    const float s1 = r + 1 < R ? w[P][r + 1 < R ? r + 1 : 0][1] : so.y;
+                    const float d0 = w[P - 1][r][0], d1 = w[P - 1][r][1], t0 = w[P + 1][r][0], t1 = w[P + 1][r][1];
+                    float res = 0.f;
+                    if (full) {
+                        const float q0 = fmaf(a.sk, ((uw + u1) + (n0 + s0)) + (d0 + t0), bv.x);
+                        const float q1 = fmaf(a.sk, ((u0 + ue) + (n1 + s1)) + (d1 + t1), bv.y);
+                        const int c = int(my >> (4 * r) & 15u) + mz;
+                        if (mx[0] + c < 7) res = fmaf(-dtab[mx[0] + c], u0, q0);
+                        if (mx[1] + c < 7) res += fmaf(-dtab[mx[1] + c], u1, q1);
+                    } else if (rows_in >> r & 1) {
+                        const Coef3* t = tab + class3(m, nz) * 16 + class3(y + r, ny) * 4;
+                        if (col0) {
+                            const Coef3* q = t + class3(x, nx);
+                            res = fmaf(-q->D, u0, general_sum(q, bv.x, uw, u1, n0, s0, d0, t0));
+                        }
+                        if (col1) {
+                            const Coef3* q = t + class3(x + 1, nx);
+                            res += fmaf(-q->D, u1, general_sum(q, bv.y, u0, ue, n1, s1, d1, t1));
+                        }
+                    }
+                    sum[r / 2] = (r & 1) ? sum[r / 2] + res : res;
+                }
+#pragma unroll
+                for (int q = 0; q < R / 2; ++q) {
+                    if ((m & 1) == 0) part[q] = sum[q];
+                    else part[q] += sum[q];
+                    const int yy = y + 2 * q;
+                    if (((m & 1) || m == nz - 1) && lane_out && (rows_out >> (2 * q) & 1))
+                        a.cb[((int64_t)(m >> 1) * a.ncy + (yy >> 1)) * a.cp + (x >> 1)] = part[q] * 0.125f;
+                }
+            }
+        }
+        if (++slot == NS) slot = 0;
     }
 }
 
+// ---------------------------------------------------------------- the small levels
+// Levels kt .. of at most kTail3 cells on copies in shared memory, one CTA: the rest of the
+// V-cycle in one launch (bound by the latency of its passes, one barrier each).
+constexpr int kTail3 = 8192, kTailThreads3 = 1024, kTailLevels3 = 14;
+
+struct Tail3 {
+    const float* b;   // right-hand side of level kt (dense rows of `pitch`)
+    float* u;         // its iterate: read if cont, written at the end
+    int pitch, nx, ny, nz, kt, nlev;
+    int nu_pre, nu_post, cont;
+    Geo3 g;
+    float alpha;
+};
+
+// Division by a small number known at run time: exact for 0 <= p, d < 2^16.
+struct SmallDiv {
+    unsigned d, m;
+    __device__ __forceinline__ explicit SmallDiv(int v) : d(v), m(v == 1 ? 0u : 0xffffffffu / (unsigned)v + 1u) {}
+    __device__ __forceinline__ int of(int p) const { return d == 1 ? p : (int)__umulhi((unsigned)p, m); }
+};
+
+struct TailLev3 {
+    float *u, *b;
+    const Coef3* tab;
+    const float *wx, *wy, *wz;  // interpolation weights toward the other coarse cell (see k3_leg)
+    int nx, ny, nz;
+};
+
+// Cell p of the half-lattice of one colour (p over ceil(nx / 2) x ny x nz); false past the row's end.
+__device__ __forceinline__ bool tail3_cell(const TailLev3& L, const SmallDiv& dx, const SmallDiv& dy, int p, int colour,
+                                           int& x, int& y, int& z) {
+    const int hx = (L.nx + 1) >> 1;
+    const int row = dx.of(p);
+    z = dy.of(row);
+    y = row - z * L.ny;
+    x = 2 * (p - row * hx) + ((y + z + colour) & 1);
+    return x < L.nx;
+}
+
+__device__ __forceinline__ float tail3_sum(const TailLev3& L, const Coef3& c, int p, int x, int y, int z, float b) {
+    const int sy = L.nx, sz = L.nx * L.ny;
+    float acc = b;
+    if (x > 0) acc = fmaf(c.cw, L.u[p - 1], acc);
+    if (x + 1 < L.nx) acc = fmaf(c.ce, L.u[p + 1], acc);
+    if (y > 0) acc = fmaf(c.cn, L.u[p - sy], acc);
+    if (y + 1 < L.ny) acc = fmaf(c.cs, L.u[p + sy], acc);
+    if (z > 0) acc = fmaf(c.cd, L.u[p - sz], acc);
+    if (z + 1 < L.nz) acc = fmaf(c.cu, L.u[p + sz], acc);
+    return acc;
+}
+
+__device__ __forceinline__ const Coef3& tail3_coef(const TailLev3& L, int x, int y, int z) {
+    return L.tab[class3(z, L.nz) * 16 + class3(y, L.ny) * 4 + class3(x, L.nx)];
+}
+
+__device__ __forceinline__ void tail3_relax(const TailLev3& L, int half_sweeps) {
+    const int n = ((L.nx + 1) >> 1) * L.ny * L.nz;
+    const SmallDiv dx((L.nx + 1) >> 1), dy(L.ny);
+    for (int h = 0; h < half_sweeps; ++h) {
+        for (int q = threadIdx.x; q < n; q += kTailThreads3) {
+            int x, y, z;
+            if (!tail3_cell(L, dx, dy, q, h & 1, x, y, z)) continue;
+            const int p = (z * L.ny + y) * L.nx + x;
+            const Coef3& c = tail3_coef(L, x, y, z);
+            L.u[p] = tail3_sum(L, c, p, x, y, z, L.b[p]) * c.iD;
+        }
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(kTailThreads3) k3_tail(const Tail3 a) {
+    extern __shared__ __align__(16) float smem3[];
+    __shared__ int off[kTailLevels3 + 1], woff[kTailLevels3 + 1];
+    Coef3* const tabs = reinterpret_cast<Coef3*>(smem3);  // 64 per level
+    float* const base = smem3 + a.nlev * 64 * (int)(sizeof(Coef3) / sizeof(float));
+    const int tid = threadIdx.x;
+    auto size = [&](int n0, int q) { return level_size(n0, a.kt + q); };
+    if (tid == 0) {
+        int o = 0, wo = 0;
+        for (int q = 0; q < a.nlev; ++q) {
+            off[q] = o;
+            woff[q] = wo;
+            o += 2 * size(a.g.n0x, q) * size(a.g.n0y, q) * size(a.g.n0z, q);
+            wo += size(a.g.n0x, q) + size(a.g.n0y, q) + size(a.g.n0z, q);
+        }
+        off[a.nlev] = o;
+        woff[a.nlev] = wo;
+    }
+    for (int t = tid; t < 64 * a.nlev; t += kTailThreads3) {
+        const int q = t >> 6, k = a.kt + q;
+        tabs[t] = table_entry(t & 63, size(a.g.n0x, q), size(a.g.n0y, q), size(a.g.n0z, q), a.g, k, a.alpha,
+                              ldexpf(1.f, -2 * k));
+    }
+    __syncthreads();
+    auto view = [&](int q) {
+        TailLev3 L;
+        L.nx = size(a.g.n0x, q);
+        L.ny = size(a.g.n0y, q);
+        L.nz = size(a.g.n0z, q);
+        L.u = base + off[q];
+        L.b = L.u + L.nx * L.ny * L.nz;
+        L.tab = tabs + 64 * q;
+        L.wx = base + off[a.nlev] + woff[q];
+        L.wy = L.wx + L.nx;
+        L.wz = L.wy + L.ny;
+        return L;
+    };
+    for (int p = tid; p < off[a.nlev]; p += kTailThreads3) base[p] = 0.f;
+    for (int q = 0; q + 1 < a.nlev; ++q) {
+        const TailLev3 L = view(q), C = view(q + 1);
+        for (int p = tid; p < L.nx + L.ny + L.nz; p += kTailThreads3) {
+            const int ax = p < L.nx ? 0 : (p < L.nx + L.ny ? 1 : 2);
+            const int i = ax == 0 ? p : (ax == 1 ? p - L.nx : p - L.nx - L.ny);
+            int I, J;
+            float w;
+            interp_axis<float>(i, ax == 0 ? a.g.n0x : (ax == 1 ? a.g.n0y : a.g.n0z), a.kt + q,
+                               ax == 0 ? C.nx : (ax == 1 ? C.ny : C.nz), I, J, w);
+            base[off[a.nlev] + woff[q] + p] = w;
+        }
+    }
+    __syncthreads();
+    {
+        const TailLev3 L = view(0);
+        for (int p = tid; p < L.nx * L.ny * L.nz; p += kTailThreads3) {
+            const int row = p / L.nx;
+            const int64_t g = (int64_t)row * a.pitch + (p - row * L.nx);
+            L.b[p] = a.b[g];
+            if (a.cont) L.u[p] = a.u[g];
+        }
+        __syncthreads();
+    }
+    for (int q = 0; q + 1 < a.nlev; ++q) {
+        const TailLev3 L = view(q), C = view(q + 1);
+        tail3_relax(L, 2 * a.nu_pre);
+        const SmallDiv dx(C.nx), dy(C.ny);
+        for (int p = tid; p < C.nx * C.ny * C.nz; p += kTailThreads3) {
+            const int row = dx.of(p), X = p - row * C.nx, Z = dy.of(row), Y = row - Z * C.ny;
+            float sum = 0.f;
+            for (int o = 0; o < 8; ++o) {
+                const int x = 2 * X + (o & 1), y = 2 * Y + ((o >> 1) & 1), z = 2 * Z + (o >> 2);
+                if (x >= L.nx || y >= L.ny || z >= L.nz) continue;
+                const int f = (z * L.ny + y) * L.nx + x;
+                const Coef3& c = tail3_coef(L, x, y, z);
+                sum += fmaf(-c.D, L.u[f], tail3_sum(L, c, f, x, y, z, L.b[f]));
+            }
+            C.b[p] = sum * 0.125f;
+        }
+        __syncthreads();
+    }
+    tail3_relax(view(a.nlev - 1), 1);  // 1 x 1 x 1: one half-sweep solves it
+    for (int q = a.nlev - 2; q >= 0; --q) {
+        const TailLev3 L = view(q), C = view(q + 1);
+        const SmallDiv dx(L.nx), dy(L.ny);
+        for (int p = tid; p < L.nx * L.ny * L.nz; p += kTailThreads3) {
+            const int row = dx.of(p), x = p - row * L.nx, z = dy.of(row), y = row - z * L.ny;
+            const float wx = L.wx[x], wy = L.wy[y], wz = L.wz[z];
+            auto other = [](int i, float w2) { return w2 == 0.f ? i >> 1 : ((i & 1) ? (i >> 1) + 1 : (i >> 1) - 1); };
+            const int Ix = x >> 1, Iy = y >> 1, Iz = z >> 1;
+            const int Jx = other(x, wx), Jy = other(y, wy), Jz = other(z, wz);
+            const float* u0 = C.u + Iz * C.ny * C.nx;
+            const float* u1 = C.u + Jz * C.ny * C.nx;
+            const float e = bilinear<float>(u0[Iy * C.nx + Ix], u0[Iy * C.nx + Jx], u0[Jy * C.nx + Ix], u0[Jy * C.nx + Jx],
+                                            wx, wy);
+            const float f = bilinear<float>(u1[Iy * C.nx + Ix], u1[Iy * C.nx + Jx], u1[Jy * C.nx + Ix], u1[Jy * C.nx + Jx],
+                                            wx, wy);
+            L.u[p] += fmaf(wz, f - e, e);
+        }
+        __syncthreads();
+        tail3_relax(L, 2 * a.nu_post);
+    }
+    const TailLev3 L = view(0);
+    for (int p = tid; p < L.nx * L.ny * L.nz; p += kTailThreads3) {
+        const int row = p / L.nx;
+        a.u[(int64_t)row * a.pitch + (p - row * L.nx)] = L.u[p];
+    }
+}
 
 // Block sum of two doubles into sums[0], sums[1] (shuffle tree, one atomic per block).
 __device__ __forceinline__ void block_sum2(double a, double b, double* sums) {
@@ -222,93 +695,213 @@ __device__ __forceinline__ void block_sum2(double a, double b, double* sums) {
     }
 }
 
-// d += e (FP64), e = the level-0 result of the last V-cycle.
-__global__ void __launch_bounds__(kThreads3) k3_update(double* __restrict__ d, const float* __restrict__ e, int64_t n) {
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x)
-        d[t] += f2d_ieee(e[t]);
+// d += e (or d = e where `first`), e = the level-0 result of the last V-cycle, over the padded rows.
+template <class D>
+__global__ void __launch_bounds__(kThreads3) k3_update(D* __restrict__ d, const float* __restrict__ e, int64_t n,
+                                                       int first) {
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
+        if constexpr (sizeof(D) == sizeof(Split) && !std::is_same<D, double>::value)
+            d[t] = first ? Split{e[t], 0.f} : split_add(d[t], e[t]);
+        else
+            d[t] = (first ? 0.0 : d[t]) + f2d_ieee(e[t]);
+    }
 }
 
-// FP64 defect pass on the finest level: r = -L_z I0 - A d (A = alpha I + L, 7-point, Neumann),
-// out = I0 + d; r goes to the level-0 right-hand side (FP32) and the level-0 iterate is zeroed
-// for the next V-cycle.  A d is formed in FP64 on the FP64 iterate (sum of the neighbours and
-// one fma with alpha + degree, where the cancellation happens), rounded once to FP32 and taken
-// from the FP32-formed -L_z I0 (exact for 8-bit input; its own rounding bounds what FP64 could
-// add there), as the slice solver's correction passes do.  sums[0] += ||r||^2 (FP64); with
-// `first` (d = 0, not read) also sums[1] += ||alpha I0 + L_xy I0||^2.  Conversions run on the
-// integer pipe.  adeg[q] = alpha + q for q = 0..6.  EXACT (tolerances below 1e-7, where the
-// FP32 rounding of the subtraction would cap the reachable residual): -L_z I0 and the
-// subtraction in FP64 too.
-template <class Tin, bool EXACT>
-__global__ void __launch_bounds__(kThreads3) k3_defect(const Tin* __restrict__ I0, const double* __restrict__ d,
-                                                       float* __restrict__ r0, float* __restrict__ u0,
-                                                       float* __restrict__ out, int nx, int ny, int nz,
-                                                       float alpha, AdegTab adeg, int first,
+// Defect pass on the finest level: r = -L_z I0 - A d (A = alpha I + L, 7-point, Neumann), out =
+// I0 + d; r goes to the level-0 right-hand side (FP32).  sums[0] += ||r||^2; with FIRST (d = 0, not
+// read) also sums[1] += ||alpha I0 + L_xy I0||^2.  Three forms of d: Split (two floats, tolerances
+// from 1e-7): A d carries the rounding errors of its sums and product and is rounded once to FP32
+// before it is taken from the FP32-formed -L_z I0 (exact for 8-bit input; its own rounding bounds
+// what more bits could add there); double with everything in FP64, -L_z I0 and the subtraction
+// included (smaller tolerances, where that rounding would cap the reachable residual).
+//
+// A thread marches along z over a chunk of kDefectZ planes of one pixel column, so that the
+// neighbours along z stay in registers; those along y and x are L1 hits of a 32 x 8 tile.  Bound
+// by instruction issue (about 130 per cell): 32 x 1024 x 1024, later passes 509 -> 190 us against
+// FP64 evaluation (bound by that pipe).
+constexpr int kDefectZ = 16;
+
+template <class D>
+struct Adeg3 {
+    D v[7];  // alpha + q, q = 0..6 (the diagonal of A for a cell with q neighbours)
+};
+
+template <class D>
+__device__ __forceinline__ D at_degree3(const Adeg3<D>& t, int q) {
+    return q == 6 ? t.v[6] : q == 5 ? t.v[5] : q == 4 ? t.v[4] : q == 3 ? t.v[3] : q == 2 ? t.v[2] : q == 1 ? t.v[1] : t.v[0];
+}
+
+// a c - (sum of the six neighbours), rounded once to binary32 (see split_apply of split.cuh).
+__device__ __forceinline__ float split_apply7(Split a, Split c, Split w, Split e, Split n, Split s, Split d, Split u) {
+    float s1, e1, s2, e2, s3, e3, s4, e4, s5, e5;
+    two_sum(w.hi, e.hi, s1, e1);
+    two_sum(n.hi, s.hi, s2, e2);
+    two_sum(d.hi, u.hi, s3, e3);
+    two_sum(s1, s2, s4, e4);
+    two_sum(s4, s3, s5, e5);
+    const float lo = (((w.lo + e.lo) + (n.lo + s.lo)) + (d.lo + u.lo)) + (((e1 + e2) + (e3 + e4)) + e5);
+    return split_finish(a, c, s5, lo);
+}
+
+template <class Tin, class D, bool FIRST>
+__global__ void __launch_bounds__(kThreads3) k3_defect(const Tin* __restrict__ I0, const D* __restrict__ d,
+                                                       float* __restrict__ r0, float* __restrict__ out, int nx, int ny,
+                                                       int nz, int pitch, float alpha, Adeg3<D> adeg,
                                                        double* __restrict__ sums) {
-    const int64_t rows = (int64_t)ny * nz, sy = nx, sz = (int64_t)nx * ny;
+    constexpr bool SPLIT = std::is_same<D, Split>::value;
+    const unsigned tx = (unsigned)((nx - 1) / 32 + 1), ty = (unsigned)((ny - 1) / 8 + 1);
+    const unsigned tile = blockIdx.x / tx, chunk = tile / ty;
+    const int x = int(blockIdx.x - tile * tx) * 32 + (threadIdx.x & 31);
+    const int y = int(tile - chunk * ty) * 8 + (threadIdx.x >> 5), zc = int(chunk) * kDefectZ;
     double rr = 0.0, bb = 0.0;
-    for (int64_t row = blockIdx.x; row < rows; row += gridDim.x)
-    for (int x = threadIdx.x; x < nx; x += blockDim.x) {
-        const int y = int(row % ny), z = int(row / ny);
-        const int64_t t = row * nx + x;
-        const bool hw = x > 0, he = x + 1 < nx, hn = y > 0, hs = y + 1 < ny, hd = z > 0, hu = z + 1 < nz;
-        const float ip = (float)I0[t];
-        // -L_z I0: the z neighbours minus the cell
-        float rhs = 0.f;
-        if (hd) rhs += (float)I0[t - sz] - ip;
-        if (hu) rhs += (float)I0[t + sz] - ip;
-        float r = rhs, o = ip;
-        double rd = 0.0;  // r in FP64 (EXACT)
-        if (EXACT) {
-            const double ipd = f2d_ieee(ip);
-            if (hd) rd += f2d_ieee((float)I0[t - sz]) - ipd;
-            if (hu) rd += f2d_ieee((float)I0[t + sz]) - ipd;
+    if (x < nx && y < ny) {
+        const int64_t sz = (int64_t)nx * ny, pz = (int64_t)pitch * ny;
+        int64_t t = ((int64_t)zc * ny + y) * nx + x, q = ((int64_t)zc * ny + y) * pitch + x;
+        const bool hw = x > 0, he = x + 1 < nx, hn = y > 0, hs = y + 1 < ny;
+        const int degxy = int(hw) + int(he) + int(hn) + int(hs);
+        float im = zc > 0 ? (float)I0[t - sz] : 0.f, ip = (float)I0[t];
+        D dm{}, dp{};
+        if (!FIRST) {
+            if (zc > 0) dm = d[q - pz];
+            dp = d[q];
         }
-        if (!first) {
-            const double dp = d[t];
-            double nb = 0.0;
-            if (hw) nb += d[t - 1];
-            if (he) nb += d[t + 1];
-            if (hn) nb += d[t - sy];
-            if (hs) nb += d[t + sy];
-            if (hd) nb += d[t - sz];
-            if (hu) nb += d[t + sz];
-            const int deg = int(hw) + int(he) + int(hn) + int(hs) + int(hd) + int(hu);
-            const double ad = deg == 6 ? adeg.v[6] : deg == 5 ? adeg.v[5] : deg == 4 ? adeg.v[4] :
-                              deg == 3 ? adeg.v[3] : deg == 2 ? adeg.v[2] : deg == 1 ? adeg.v[1] : adeg.v[0];
-            const double Ad = fma(ad, dp, -nb);
-            if (EXACT) {
-                rd -= Ad;
-                r = d2f_ieee(rd);
+        float rs = 0.f, bs = 0.f;  // FP32 sums of at most kDefectZ squares
+        const int ze = min(zc + kDefectZ, nz);
+        for (int z = zc; z < ze; ++z, t += sz, q += pz) {
+            const bool hd = z > 0, hu = z + 1 < nz;
+            const float in = hu ? (float)I0[t + sz] : 0.f;
+            // -L_z I0: the z neighbours minus the cell
+            float rhs = 0.f;
+            if (hd) rhs += im - ip;
+            if (hu) rhs += in - ip;
+            float r = rhs, o = ip;
+            if (!FIRST) {
+                const D zero{};
+                const D dn = hu ? d[q + pz] : zero;
+                const D w = hw ? d[q - 1] : zero, e = he ? d[q + 1] : zero;
+                const D n = hn ? d[q - pitch] : zero, s = hs ? d[q + pitch] : zero;
+                const D a = at_degree3(adeg, degxy + int(hd) + int(hu));
+                if constexpr (SPLIT) {
+                    r = rhs - split_apply7(a, dp, w, e, n, s, dm, dn);
+                    o = ip + dp.hi;
+                } else {
+                    const double id = f2d_ieee(ip);
+                    double rd = 0.0;
+                    if (hd) rd += f2d_ieee(im) - id;
+                    if (hu) rd += f2d_ieee(in) - id;
+                    rd -= fma(a, dp, -((((w + e) + n) + s) + (dm + dn)));
+                    r = d2f_ieee(rd);
+                    rr = fma(rd, rd, rr);
+                    o = ip + d2f_ieee(dp);
+                }
+                dm = dp;
+                dp = dn;
             } else {
-                r = rhs - d2f_ieee(Ad);
+                float lxy = 0.f;  // L_xy I0
+                if (hw) lxy += ip - (float)I0[t - 1];
+                if (he) lxy += ip - (float)I0[t + 1];
+                if (hn) lxy += ip - (float)I0[t - nx];
+                if (hs) lxy += ip - (float)I0[t + nx];
+                const float b = fmaf(alpha, ip, lxy);
+                bs = fmaf(b, b, bs);
             }
-            o = ip + d2f_ieee(dp);
-        } else {
-            float lxy = 0.f;  // L_xy I0
-            if (hw) lxy += ip - (float)I0[t - 1];
-            if (he) lxy += ip - (float)I0[t + 1];
-            if (hn) lxy += ip - (float)I0[t - sy];
-            if (hs) lxy += ip - (float)I0[t + sy];
-            const double b = f2d_ieee(fmaf(alpha, ip, lxy));
-            bb = fma(b, b, bb);
+            if (SPLIT || FIRST) rs = fmaf(r, r, rs);
+            r0[q] = r;
+            out[t] = o;
+            im = ip;
+            ip = in;
         }
-        if (!EXACT) rd = f2d_ieee(r);
-        rr = fma(rd, rd, rr);
-        r0[t] = r;
-        u0[t] = 0.f;
-        out[t] = o;
+        rr += f2d_ieee(rs);
+        bb += f2d_ieee(bs);
     }
     block_sum2(rr, bb, sums);
 }
 
-// Blocks for a pass over `rows` rows of `nx` cells: one block per row (threads across the
-// row), at most 16 per SM; blocks loop over rows.
-unsigned grid_rows(int64_t rows) {
-    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(rows, (int64_t)kNumSMs * 16));
-}
 unsigned grid_for(int64_t n) {
     const int64_t blocks = (n + kThreads3 - 1) / kThreads3;
     return (unsigned)std::max<int64_t>(1, std::min<int64_t>(blocks, (int64_t)kNumSMs * 16));
+}
+
+}  // namespace
+
+namespace {
+
+// Sweeps of the kernels of one leg: an odd number of passes of at most two sweeps each (a leg
+// reads one iterate buffer and ends in the other; see gd_multigrid).
+std::vector<int> leg_sweeps(int nu) {
+    int n = std::max(1, (nu + 1) / 2);
+    if (n % 2 == 0) ++n;
+    std::vector<int> v(n, 1);
+    if (nu == 0) v[0] = 0;
+    for (int i = 0; i < nu - n; ++i) v[i] = 2;
+    return v;
+}
+
+template <int S, bool ZERO, bool UP>
+int launch_leg3_one(const Leg3& a, dim3 grid, cudaStream_t st) {
+    static std::mutex mu;
+    static bool done[64] = {false};
+    int dev = 0;
+    EMF_CUDA(cudaGetDevice(&dev));
+    if (dev >= 0 && dev < 64) {
+        std::lock_guard<std::mutex> lk(mu);
+        if (!done[dev]) {
+            EMF_CUDA(cudaFuncSetAttribute(k3_leg<S, ZERO, UP>, cudaFuncAttributeMaxDynamicSharedMemorySize, leg3_smem<S>()));
+            done[dev] = true;
+        }
+    }
+    k3_leg<S, ZERO, UP><<<grid, kWarps3 * 32, leg3_smem<S>(), st>>>(a);
+    EMF_CHECK_LAUNCH();
+    return EMFUSE_OK;
+}
+
+template <int S>
+int launch_leg3_s(const Leg3& a, bool zero, bool up, dim3 grid, cudaStream_t st) {
+    if (up) return launch_leg3_one<S, false, true>(a, grid, st);
+    if (zero) return launch_leg3_one<S, true, false>(a, grid, st);
+    return launch_leg3_one<S, false, false>(a, grid, st);
+}
+
+// One pass of `sweeps` sweeps (0, 1 or 2) over a level.
+int launch_leg3(Leg3 a, int sweeps, bool zero, bool up, const char* name, double bytes, cudaStream_t st) {
+    const int halo = 2 * sweeps + (a.cb ? 1 : 0);
+    a.halo = (halo + 1) / 2 * 2;
+    const int ox = kTile3 - 2 * a.halo;
+    const int64_t tx = ceil_div(a.nx, ox), ty = ceil_div(a.ny, ox);
+    // one chunk along z, unless the tiles leave SMs idle: then chunks of at least 8 planes (each
+    // end of a chunk recomputes 2 * sweeps planes)
+    const int64_t chunks = std::max<int64_t>(1, std::min<int64_t>(kNumSMs / (tx * ty), a.nz / 8));
+    a.zch = (int)round_up(ceil_div(a.nz, chunks), 2);
+    const int64_t cz = ceil_div(a.nz, a.zch);
+    a.tx = (unsigned)tx;
+    a.ty = (unsigned)ty;
+    const dim3 grid((unsigned)(tx * ty * cz));
+    KernelScope ks(name, st, bytes);
+    switch (sweeps) {
+        case 0: return launch_leg3_s<0>(a, zero, up, grid, st);
+        case 1: return launch_leg3_s<2>(a, zero, up, grid, st);
+        default: return launch_leg3_s<4>(a, zero, up, grid, st);
+    }
+}
+
+// cells and sides: summed over the tail's levels
+int launch_tail3(const Tail3& a, size_t cells, size_t sides, cudaStream_t st) {
+    const int smem = a.nlev * 64 * (int)sizeof(Coef3) + (int)((2 * cells + sides) * sizeof(float));
+    static std::mutex mu;
+    static int set[64] = {0};
+    int dev = 0;
+    EMF_CUDA(cudaGetDevice(&dev));
+    if (dev >= 0 && dev < 64) {
+        std::lock_guard<std::mutex> lk(mu);
+        if (set[dev] < smem) {
+            EMF_CUDA(cudaFuncSetAttribute(k3_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+            set[dev] = smem;
+        }
+    }
+    KernelScope ks("gd3_tail", st, 8.0 * (double)cells);
+    k3_tail<<<1, kTailThreads3, smem, st>>>(a);
+    EMF_CHECK_LAUNCH();
+    return EMFUSE_OK;
 }
 
 }  // namespace
@@ -317,107 +910,176 @@ int gd_multigrid(const void* in, int dt, float* out, int64_t nx, int64_t ny, int
                  const emfuse_solve_opts& opts, emfuse_slice_stats* stats, cudaStream_t st) {
     // levels: ceil halving per axis down to 1 x 1 x 1
     std::vector<Lev3> lev;
-    {
-        int k = 0;
-        for (;; ++k) {
-            Lev3 L{};
-            L.nx = (int)(((nx - 1) >> k) + 1);
-            L.ny = (int)(((ny - 1) >> k) + 1);
-            L.nz = (int)(((nz - 1) >> k) + 1);
-            lev.push_back(L);
-            if (L.nx == 1 && L.ny == 1 && L.nz == 1) break;
-        }
+    for (int k = 0;; ++k) {
+        Lev3 L{};
+        L.nx = level_size((int)nx, k);
+        L.ny = level_size((int)ny, k);
+        L.nz = level_size((int)nz, k);
+        L.pitch = (int)round_up(L.nx, 2);
+        lev.push_back(L);
+        if (L.nx == 1 && L.ny == 1 && L.nz == 1) break;
     }
     const int nlev = (int)lev.size();
-    size_t cells = 0;
-    for (const auto& L : lev) cells += (size_t)L.nx * L.ny * L.nz;
-    const int64_t n0 = nx * ny * nz;
-    DeviceBuffer ub, bbuf, dbuf, sums;
-    EMF_TRY(ub.alloc(cells * sizeof(float), st));
-    EMF_TRY(bbuf.alloc(cells * sizeof(float), st));
-    EMF_TRY(dbuf.alloc((size_t)n0 * sizeof(double), st));
-    EMF_TRY(sums.alloc(2 * sizeof(double), st));
-    {
-        size_t off = 0;
-        for (auto& L : lev) {
-            L.u = ub.as<float>() + off;
-            L.b = bbuf.as<float>() + off;
-            off += (size_t)L.nx * L.ny * L.nz;
+    auto padded = [&](int k) { return (size_t)lev[k].pitch * lev[k].ny * lev[k].nz; };
+    auto cells = [&](int k) { return (size_t)lev[k].nx * lev[k].ny * lev[k].nz; };
+    int kt = 0;  // first level of the tail kernel
+    while (cells(kt) > (size_t)kTail3) ++kt;
+    size_t tail_cells = 0, tail_sides = 0, all = 0;
+    for (int k = 0; k < nlev; ++k) {
+        all += padded(k);
+        if (k >= kt) {
+            tail_cells += cells(k);
+            tail_sides += (size_t)lev[k].nx + lev[k].ny + lev[k].nz;
         }
     }
-    EMF_CUDA(cudaMemsetAsync(dbuf.as<double>(), 0, (size_t)n0 * sizeof(double), st));  // d = 0
+    const size_t coarse = all - padded(0), n0p = padded(0);
+    const bool split = opts.tol >= 1e-7;
+    // Iterate buffers.  A leg reads one buffer and ends in the other: DOWN u -> v (from u only when
+    // a V-cycle continues from the last one), UP v -> u.  The finest level's v is the caller's
+    // `out`, which every defect pass rewrites; and between its two legs the finest level's u is
+    // free and holds the v of the coarse levels.
+    DeviceBuffer ub, bbuf, dbuf, sums;
+    EMF_TRY(ub.alloc((std::max(n0p, coarse) + coarse) * sizeof(float), st));
+    EMF_TRY(bbuf.alloc(all * sizeof(float), st));
+    EMF_TRY(dbuf.alloc(n0p * sizeof(double), st));
+    EMF_TRY(sums.alloc(2 * sizeof(double), st));
+    {
+        float *u = ub.as<float>() + std::max(n0p, coarse), *v = ub.as<float>(), *b = bbuf.as<float>();
+        for (int k = 0; k < nlev; ++k) {
+            lev[k].b = b;
+            b += padded(k);
+            lev[k].u = k == 0 ? ub.as<float>() : u;
+            lev[k].v = k == 0 ? out : v;
+            lev[k].vpitch = k == 0 ? (int)nx : lev[k].pitch;
+            if (k > 0) {
+                u += padded(k);
+                v += padded(k);
+            }
+        }
+    }
     const Geo3 g{(int)nx, (int)ny, (int)nz};
     const float af = (float)alpha;
-    double* d = dbuf.as<double>();
-    double* hs = nullptr;  // pinned copy of the norms
-    EMF_CUDA(cudaMallocHost(&hs, 2 * sizeof(double)));
-    struct HostFree {
-        double* p;
-        ~HostFree() { cudaFreeHost(p); }
-    } hs_guard{hs};
+    void* const d = dbuf.as<void>();
 
-    auto defect = [&](int first) -> int {
+    double hs[2] = {0.0, 0.0};
+    auto defect = [&](bool first) -> int {
         EMF_CUDA(cudaMemsetAsync(sums.as<double>(), 0, 2 * sizeof(double), st));
-        KernelScope ks("gd3_defect", st, (double)n0 * ((dt == EMFUSE_U8 ? 1.0 : 4.0) + (first ? 0.0 : 8.0) + 12.0),
-                       first ? 0.0 : (double)n0 * 8.0);
-        AdegTab adeg;
-        for (int q = 0; q <= 6; ++q) adeg.v[q] = alpha + (double)q;
-        const bool exact = opts.tol < 1e-7;
-        const unsigned gr = grid_rows(ny * nz);
-#define EMF_GD3_DEFECT(TT, EX)                                                                            \
-    k3_defect<TT, EX><<<gr, kThreads3, 0, st>>>((const TT*)in, d, lev[0].b, lev[0].u, out, (int)nx, (int)ny, \
-                                                (int)nz, af, adeg, first, sums.as<double>())
-        if (dt == EMFUSE_U8) {
-            if (exact) EMF_GD3_DEFECT(uint8_t, true);
-            else EMF_GD3_DEFECT(uint8_t, false);
-        } else {
-            if (exact) EMF_GD3_DEFECT(float, true);
-            else EMF_GD3_DEFECT(float, false);
+        {
+            const double n0 = (double)nx * ny * nz;
+            KernelScope ks("gd3_defect", st, n0 * ((dt == EMFUSE_U8 ? 1.0 : 4.0) + (first ? 0.0 : 8.0) + 8.0),
+                           first || split ? 0.0 : n0 * 8.0);
+            const unsigned grid = (unsigned)(ceil_div(nx, 32) * ceil_div(ny, 8) * ceil_div(nz, kDefectZ));
+            auto run = [&](auto tin, auto dd, auto first_tag) {
+                using Tin = decltype(tin);
+                using D = decltype(dd);
+                Adeg3<D> adeg;
+                for (int q = 0; q <= 6; ++q) {
+                    const double v = alpha + (double)q;
+                    if constexpr (std::is_same<D, Split>::value) {
+                        adeg.v[q].hi = (float)v;
+                        adeg.v[q].lo = (float)(v - (double)adeg.v[q].hi);
+                    } else {
+                        adeg.v[q] = v;
+                    }
+                }
+                k3_defect<Tin, D, decltype(first_tag)::value><<<grid, kThreads3, 0, st>>>(
+                    (const Tin*)in, (const D*)d, lev[0].b, out, (int)nx, (int)ny, (int)nz, lev[0].pitch, af, adeg,
+                    sums.as<double>());
+            };
+            auto run_d = [&](auto tin) {
+                if (first) run(tin, Split{}, std::true_type{});
+                else if (split) run(tin, Split{}, std::false_type{});
+                else run(tin, 0.0, std::false_type{});
+            };
+            if (dt == EMFUSE_U8) run_d(uint8_t{});
+            else run_d(float{});
+            EMF_CHECK_LAUNCH();
         }
-#undef EMF_GD3_DEFECT
-        EMF_CHECK_LAUNCH();
         EMF_CUDA(cudaMemcpyAsync(hs, sums.as<double>(), 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
         EMF_CUDA(cudaStreamSynchronize(st));
         return EMFUSE_OK;
     };
-    // interior diagonal of level k: coef3's formula with unit widths and faces
-    auto diag = [&](int k) {
-        const float sk = std::ldexp(1.f, -2 * k);
-        Diag3 di;
-        di.D = std::fmaf(af, 1.f, ((sk + sk) + (sk + sk)) + (sk + sk));
-        di.iD = (float)(1.0 / (double)di.D);
-        return di;
-    };
-    auto relax = [&](int k, int sweeps) -> int {
-        const Lev3& L = lev[k];
-        const float sk = std::ldexp(1.f, -2 * k);
-        const int64_t n = (int64_t)L.ny * L.nz;  // rows
-        for (int s = 0; s < sweeps; ++s)
-            for (int colour = 0; colour < 2; ++colour) {
-                KernelScope ks(k == 0 ? "gd3_relax_l0" : "gd3_relax", st, (double)L.nx * L.ny * L.nz * 6.0);
-                k3_relax<<<grid_rows(n), kThreads3, 0, st>>>(L, g, k, af, sk, diag(k), colour);
-                EMF_CHECK_LAUNCH();
+    auto vec = [](const float* p, int pitch) { return pitch % 2 == 0 && (reinterpret_cast<uintptr_t>(p) & 7) == 0 ? 1 : 0; };
+    const std::vector<int> dn = leg_sweeps(opts.nu_pre), up = leg_sweeps(opts.nu_post);
+    // One V-cycle from zero or (cont) from the last result; `add`: the result is added to d (or
+    // becomes it, d_first) instead of staying in lev[0].u.
+    auto vcycle = [&](bool cont, bool add, bool d_first) -> int {
+        auto leg = [&](int k) {
+            const Lev3& F = lev[k];
+            Leg3 a{};
+            a.b = F.b;
+            a.bp = F.pitch;
+            a.nx = F.nx;
+            a.ny = F.ny;
+            a.nz = F.nz;
+            a.k = k;
+            a.g = g;
+            a.alpha = af;
+            a.sk = std::ldexp(1.f, -2 * k);
+            if (k + 1 < nlev) {
+                a.ncx = lev[k + 1].nx;
+                a.ncy = lev[k + 1].ny;
+                a.ncz = lev[k + 1].nz;
+                a.cp = lev[k + 1].pitch;
             }
-        return EMFUSE_OK;
-    };
-    auto vcycle = [&]() -> int {
-        for (int k = 0; k + 1 < nlev; ++k) {
-            EMF_TRY(relax(k, opts.nu_pre));
-            const Lev3 &F = lev[k], &C = lev[k + 1];
-            KernelScope ks(k == 0 ? "gd3_restrict_l0" : "gd3_restrict", st, (double)F.nx * F.ny * F.nz * 8.0);
-            k3_residual_restrict<<<grid_rows((int64_t)C.ny * C.nz), kThreads3, 0, st>>>(
-                F, C, g, k, af, std::ldexp(1.f, -2 * k), diag(k));
-            EMF_CHECK_LAUNCH();
+            return a;
+        };
+        // pass i of a leg: odd passes u -> v (DOWN) or v -> u (UP), the others back
+        auto buffers = [&](Leg3& a, int k, bool from_u) {
+            const Lev3& F = lev[k];
+            a.src = from_u ? F.u : F.v;
+            a.sp = from_u ? F.pitch : F.vpitch;
+            a.dst = from_u ? F.v : F.u;
+            a.dp = from_u ? F.vpitch : F.pitch;
+            a.svec = vec(a.src, a.sp);
+            a.dvec = vec(a.dst, a.dp);
+        };
+        for (int k = 0; k < kt; ++k) {
+            for (size_t i = 0; i < dn.size(); ++i) {
+                Leg3 a = leg(k);
+                buffers(a, k, i % 2 == 0);
+                const bool zero = i == 0 && !(cont && k == 0), last = i + 1 == dn.size();
+                if (last) a.cb = lev[k + 1].b;
+                EMF_TRY(launch_leg3(a, dn[i], zero, false, k == 0 ? "gd3_down_l0" : "gd3_down",
+                                    (double)cells(k) * ((zero ? 8.0 : 12.0) + (last ? 0.5 : 0.0)), st));
+            }
         }
-        EMF_TRY(relax(nlev - 1, 1));  // 1 x 1 x 1: one half-sweep solves it
-        for (int k = nlev - 2; k >= 0; --k) {
-            const Lev3 &F = lev[k], &C = lev[k + 1];
-            {
-                KernelScope ks(k == 0 ? "gd3_prolong_l0" : "gd3_prolong", st, (double)F.nx * F.ny * F.nz * 8.0);
-                k3_prolong_add<<<grid_rows((int64_t)F.ny * F.nz), kThreads3, 0, st>>>(F, C, g, k);
-                EMF_CHECK_LAUNCH();
+        {
+            Tail3 t{};
+            t.b = lev[kt].b;
+            t.u = lev[kt].u;
+            t.pitch = lev[kt].pitch;
+            t.nx = lev[kt].nx;
+            t.ny = lev[kt].ny;
+            t.nz = lev[kt].nz;
+            t.kt = kt;
+            t.nlev = nlev - kt;
+            t.nu_pre = opts.nu_pre;
+            t.nu_post = opts.nu_post;
+            t.cont = cont && kt == 0;
+            t.g = g;
+            t.alpha = af;
+            EMF_TRY(launch_tail3(t, tail_cells, tail_sides, st));
+        }
+        for (int k = kt - 1; k >= 0; --k)
+            for (size_t i = 0; i < up.size(); ++i) {
+                Leg3 a = leg(k);
+                buffers(a, k, i % 2 != 0);
+                if (i == 0) a.cu = lev[k + 1].u;
+                if (k == 0 && add && split && i + 1 == up.size()) {
+                    a.d = (Split*)d;
+                    a.pitch_d = lev[0].pitch;
+                    a.d_first = d_first;
+                }
+                EMF_TRY(launch_leg3(a, up[i], false, true, k == 0 ? "gd3_up_l0" : "gd3_up",
+                                    (double)cells(k) * (8.0 + (a.d ? (d_first ? 8.0 : 16.0) : 4.0) + (i == 0 ? 0.5 : 0.0)),
+                                    st));
             }
-            EMF_TRY(relax(k, opts.nu_post));
+        if (add && (kt == 0 || !split)) {
+            KernelScope ks("gd3_update", st, (double)n0p * (d_first ? 12.0 : 20.0));
+            if (split) k3_update<Split><<<grid_for((int64_t)n0p), kThreads3, 0, st>>>((Split*)d, lev[0].u, (int64_t)n0p, d_first);
+            else k3_update<double><<<grid_for((int64_t)n0p), kThreads3, 0, st>>>((double*)d, lev[0].u, (int64_t)n0p, d_first);
+            EMF_CHECK_LAUNCH();
         }
         return EMFUSE_OK;
     };
@@ -427,27 +1089,20 @@ int gd_multigrid(const void* in, int dt, float* out, int64_t nx, int64_t ny, int
         if (!std::isfinite(hs[0]) || !std::isfinite(bnorm)) return std::nan("");
         return bnorm > 0.0 ? std::sqrt(hs[0]) / bnorm : (hs[0] > 0.0 ? HUGE_VAL : 0.0);
     };
-    EMF_TRY(defect(1));
+    EMF_TRY(defect(true));
     const double bnorm = std::sqrt(hs[1]);
     double rel = relres(bnorm);
     int v = 0;
     bool finite = std::isfinite(rel);
     while (finite && rel > opts.tol && v < opts.max_vcycles) {
-        EMF_TRY(vcycle());
-        // before the first FP64 pass, further FP32 V-cycles continue from the last iterate
-        // (their fine residual is formed in FP32 inside the cycle), as in the slice solver
-        if (v == 0)
-            for (int extra = 1; extra < opts.first_vcycles && extra < opts.max_vcycles; ++extra, ++v)
-                EMF_TRY(vcycle());
-        {
-            KernelScope ks("gd3_update", st, (double)n0 * 20.0);
-            k3_update<<<grid_for(n0), kThreads3, 0, st>>>(d, lev[0].u, n0);
-            EMF_CHECK_LAUNCH();
-        }
-        EMF_TRY(defect(0));
+        // before the first defect pass, further FP32 V-cycles continue from the last iterate (their
+        // fine residual is formed in FP32 inside the cycle), as in the slice solver
+        const bool first = v == 0;
+        const int n = first ? std::max(1, std::min(opts.first_vcycles, opts.max_vcycles)) : 1;
+        for (int i = 0; i < n; ++i, ++v) EMF_TRY(vcycle(i > 0, i + 1 == n, first));
+        EMF_TRY(defect(false));
         rel = relres(bnorm);
         finite = std::isfinite(rel);
-        ++v;
     }
     if (stats) {
         stats->vcycles = v;
