@@ -28,14 +28,16 @@
 #include <cstring>
 #include <map>
 #include <memory>
-#include <tuple>
 #include <mutex>
+#include <tuple>
+#include <type_traits>
 #include <vector>
 
 #include "emfuse_common.cuh"
 #include "emfuse_internal.cuh"
 #include "fpconv.cuh"
 #include "mg_fused.cuh"
+#include "split.cuh"
 #include "tma.cuh"
 
 namespace emfuse {
@@ -145,9 +147,18 @@ struct TopSlice {
 template <class TF>
 struct AlphaDeg {
     TF v[5];
+    Split s[5];     // the same, split
     float alpha_f;  // alpha rounded to float once on the host (a conversion per thread would
                     // take the FP64 pipe)
 };
+
+// t[deg] without indexing a kernel parameter at run time (which would copy it to local memory)
+template <class E>
+__device__ __forceinline__ E at_degree(const E (&t)[5], int deg) {
+    return deg == 4 ? t[4] : (deg == 3 ? t[3] : (deg == 2 ? t[2] : (deg == 1 ? t[1] : t[0])));
+}
+__device__ __forceinline__ Split as_split(float v) { return Split{v, 0.f}; }
+__device__ __forceinline__ Split as_split(Split v) { return v; }
 
 // Device-side state of the outer loop of one solve (one per plan).  The loop (residual pass,
 // convergence check, V-cycle, residual pass, ...) is decided on the device by k_check after
@@ -173,7 +184,7 @@ struct CallPtrs {
 };
 
 constexpr int kTopTX = 64;
-constexpr int kTopTY = 32;  // two rows of 4 cells per thread; the one-cell halo of d is 9 % extra
+constexpr int kTopTY = 32;  // 8 cells per thread; the one-cell halo of d is 9 % extra
 
 // MODE 0: d = 0, r = alpha (s - o)          (first residual; also accumulates ||b||^2)
 // MODE 1: d_new = e                          (first correction)
@@ -182,13 +193,24 @@ constexpr int kTopTY = 32;  // two rows of 4 cells per thread; the one-cell halo
 // residual this pass measures, so the output is always the latest iterate).
 // d_old and d_new are different buffers (they alternate between passes): a tile reads d_old
 // and e on a one-cell halo while its neighbours write d_new.  Arithmetic on d and r in TF
-// (FP64 when mixed); the FP64 work per cell is the 5-point operator on d (and in MODE 2 the
-// update d_old + e).  Conversions between TV and TF run on the integer pipe (fpconv.cuh).
-template <class TF, class TV, class To, int MODE, bool EXACT>
-__global__ void __launch_bounds__(256)
+// (FP64 when mixed).  Conversions between TV and TF run on the integer pipe (fpconv.cuh).
+//
+// Mixed precision, three forms (FORM): kExact (tolerances below 1e-7) subtracts in FP64 too.
+// Otherwise A d is rounded to FP32 before the subtraction, and large batches (kSplit) need not
+// form it in FP64: the tile holds the FP64 values split into two floats (48 bits) and A d is
+// evaluated from those on the FP32 pipe (split.cuh), off by about 2^-46 of the largest value
+// before that rounding.  The iterate itself stays in FP64; what is left for the FP64 pipe is the
+// update d_old + e of MODE 2 (the first correction has none), and the pass is bound by memory
+// instead.  64 x 2048 x 2048, first and later correction together: 4.93 -> 3.50 ms (ragged batch of
+// 291 M cells 7.04 -> 4.82), the first residual 0.73 -> 0.59.  64 warps per SM hide the loads: at 48
+// warps the split passes take 4.17 ms, at 32 5.69.
+enum : int { kRounded = 0, kExact = 1, kSplit = 2 };
+
+template <class TF, class TV, class To, int MODE, int FORM>
+__global__ void __launch_bounds__(256, MODE == 0 ? 6 : 8)
 k_top(const TopSlice* __restrict__ top, const int64_t* __restrict__ tile_start, int nslices,
       const int* __restrict__ active, const CallPtrs* __restrict__ call, const SolveState* __restrict__ state,
-      TF* __restrict__ dbuf0, TF* __restrict__ dbuf1, double alpha, AlphaDeg<TF> ad,
+      TF* __restrict__ dbuf0, TF* __restrict__ dbuf1, AlphaDeg<TF> ad,
       double* __restrict__ norms) {
     const int64_t t = blockIdx.x;
     const int j = find_item_warp(tile_start, nslices, t);
@@ -210,82 +232,141 @@ k_top(const TopSlice* __restrict__ top, const int64_t* __restrict__ tile_start, 
     const int tid = threadIdx.x;
     const TV* e = static_cast<const TV*>(G.u0);
     TV* r0 = static_cast<TV*>(G.b0);
-    __shared__ TF dsm[kTopTY + 2][kTopTX + 2];
-    if (MODE >= 1) {
-        for (int q = tid; q < (kTopTY + 2) * (kTopTX + 2); q += 256) {
-            const int rr = q / (kTopTX + 2), cc = q - rr * (kTopTX + 2);
-            const int gx = tx0 - 1 + cc, gy = ty0 - 1 + rr;
-            TF v = TF(0);
-            if (gx >= 0 && gx < G.nx && gy >= 0 && gy < G.ny) {
-                const TF ev = cvt<TF>(e[(int64_t)gy * G.pitch0 + gx]);
-                v = MODE == 1 ? ev : d_old[G.off + (int64_t)gy * G.nx + gx] + ev;
-            }
-            dsm[rr][cc] = v;
-        }
-        __syncthreads();
-    }
+    constexpr bool SPLIT = FORM == kSplit && MODE >= 1;
+    // staged values; in MODE 1 they are FP32 numbers
+    using TS = typename std::conditional<!SPLIT, TF, typename std::conditional<MODE == 1, float, Split>::type>::type;
+    __shared__ TS dsm[kTopTY + 2][kTopTX + 2];
+    // a thread's 8 cells: columns lane and lane + 32 of rows warp, warp + 8, + 16, + 24, so that a
+    // warp reads and writes whole lines; offsets from the tile's corner fit an int
+    const int lane = tid & 31, warp = tid >> 5, nx = G.nx;
+    const int64_t corner = G.off + (int64_t)ty0 * nx + tx0, corner0 = (int64_t)ty0 * G.pitch0 + tx0;
+    const float *sT = rhs ? rhs + corner : s + corner;
+    const To* oT = o + corner;
+    const TV* eT = e + corner0;
+    TV* rT = r0 + corner0;
+    const TF* dT = d_old + corner;
+    TF* nT = d_new + corner;
+    float* outT = out + corner;
     const float af = ad.alpha_f;
     // squared norms: FP32 partial sums over a warp's 256 cells, FP64 from there on (per-block
     // sums, per-slice atomics); this keeps the FP64 pipe for the residual itself
     float rrf = 0.f, bbf = 0.f;
+    // the pass over the tile; INNER: the tile and its halo lie inside the slice
+    auto pass = [&](auto inner_tag) {
+        constexpr bool INNER = decltype(inner_tag)::value;
+        auto inside = [&](int lx, int ly) { return INNER || (tx0 + lx < nx && ty0 + ly < G.ny); };
+        // the correction passes run 64 warps per SM at 32 registers; the first residual, without
+        // staged values, has registers to load its 8 cells before it uses any
+        constexpr int kUnroll = SPLIT || MODE == 0 ? 8 : 2;
+        constexpr int kAhead = MODE == 0 ? 8 : 1;
+        float sva[kAhead], ova[kAhead];
+        if (MODE == 0) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int ly = tid / 16 + 16 * (i >> 2);  // rows tid / 16 and tid / 16 + 16
-        const int y = ty0 + ly;
-        const int lx = (tid % 16) + 16 * (i & 3);  // consecutive threads, consecutive cells
-        const int x = tx0 + lx;
-        if (x >= G.nx || y >= G.ny) continue;
-        const int64_t p = G.off + (int64_t)y * G.nx + x;
-        const bool hw = x > 0, he = x + 1 < G.nx, hn = y > 0, hs = y + 1 < G.ny;
-        float bc, ov = 0.f;
-        if (rhs) {
-            bc = rhs[p];
-            if (MODE == 0) bbf = fmaf(bc, bc, bbf);
-        } else {
-            const float sv = s[p];
-            ov = float(o[p]);
-            bc = af * (sv - ov);
-            if (MODE == 0) {
-                // ||b||^2 with b = alpha s + L o, for the relative-residual denominator
-                float lo = 0.f;
-                if (hw) lo += ov - float(o[p - 1]);
-                if (he) lo += ov - float(o[p + 1]);
-                if (hn) lo += ov - float(o[p - G.nx]);
-                if (hs) lo += ov - float(o[p + G.nx]);
-                const float b = fmaf(af, sv, lo);
-                bbf = fmaf(b, b, bbf);
+            for (int i = 0; i < kAhead; ++i) {
+                const int lx = lane + 32 * (i & 1), ly = warp + 8 * (i >> 1);
+                sva[i] = ova[i] = 0.f;
+                if (inside(lx, ly)) {
+                    sva[i] = sT[ly * nx + lx];
+                    if (!rhs) ova[i] = float(oT[ly * nx + lx]);
+                }
             }
         }
-        TV rv;
-        if (MODE == 0) {
-            rv = cvt<TV>(bc);
-        } else {
-            const TF c = dsm[ly + 1][lx + 1];
-            const TF nsum = (dsm[ly + 1][lx] + dsm[ly + 1][lx + 2]) + (dsm[ly][lx + 1] + dsm[ly + 2][lx + 1]);
-            const int deg = int(hw) + int(he) + int(hn) + int(hs);
-            const TF adeg = deg == 4 ? ad.v[4] : (deg == 3 ? ad.v[3] : (deg == 2 ? ad.v[2] : (deg == 1 ? ad.v[1] : ad.v[0])));
-            // A d in TF (FP64 when mixed): the operator on the high-precision iterate, where
-            // the cancellation between alpha d + L d and the right-hand side happens
-            const TF Ad = fma_t(adeg, c, -nsum);
-            // r = bc - A d.  bc = alpha (s - o) is formed in FP32, so its own rounding (~6e-8
-            // |bc|) bounds what FP64 could add here: unless EXACT, A d is rounded to the
-            // V-cycle type before the subtraction (same order of error, one FP64 operation per
-            // cell less).  That caps the reachable relative residual near 6e-8 ||bc|| / ||b||;
-            // tolerances below 1e-7 select EXACT.
-            if constexpr (!EXACT && sizeof(TV) < sizeof(TF)) rv = bc - cvt<TV>(Ad);
-            else rv = cvt<TV>(cvt<TF>(bc) - Ad);
-            d_new[p] = c;
-            // output: d alone in the adjoint mode, else o + d (in FP64 when TV is FP64)
-            float f;
-            if (rhs) f = cvt<float>(c);
-            else if constexpr (sizeof(TV) == 8) f = cvt<float>(cvt<double>(ov) + c);
-            else f = ov + cvt<float>(c);
-            out[p] = f;
+        if (MODE >= 1) {
+            // the iterate at a cell (halo included)
+            auto iterate = [&](int lx, int ly) -> TF {
+                const TF ev = cvt<TF>(eT[ly * G.pitch0 + lx]);
+                return MODE == 1 ? ev : dT[ly * nx + lx] + ev;
+            };
+            auto staged = [&](int lx, int ly, TF v) -> TS {
+                if constexpr (!SPLIT) return v;
+                else if constexpr (MODE == 1) return eT[ly * G.pitch0 + lx];
+                else return split_of(v);
+            };
+#pragma unroll kUnroll
+            for (int i = 0; i < 8; ++i) {
+                const int lx = lane + 32 * (i & 1), ly = warp + 8 * (i >> 1);
+                TS c = TS{};
+                if (inside(lx, ly)) {
+                    const TF v = iterate(lx, ly);
+                    c = staged(lx, ly, v);
+                    nT[ly * nx + lx] = v;
+                }
+                dsm[ly + 1][lx + 1] = c;
+            }
+            if (tid < 2 * (kTopTX + kTopTY)) {  // the halo's two rows, then its two columns
+                const bool row = tid < 2 * kTopTX;
+                const int q = row ? tid : tid - 2 * kTopTX;
+                const int lx = row ? q % kTopTX : (q < kTopTY ? -1 : kTopTX);
+                const int ly = row ? (q < kTopTX ? -1 : kTopTY) : q % kTopTY;
+                const int gx = tx0 + lx, gy = ty0 + ly;
+                TS v = TS{};
+                if (INNER || (gx >= 0 && gx < nx && gy >= 0 && gy < G.ny)) v = staged(lx, ly, iterate(lx, ly));
+                dsm[ly + 1][lx + 1] = v;
+            }
+            __syncthreads();
         }
-        r0[(int64_t)y * G.pitch0 + x] = rv;
-        const float rf = cvt<float>(rv);
-        rrf = fmaf(rf, rf, rrf);
-    }
+#pragma unroll kUnroll
+        for (int i = 0; i < 8; ++i) {
+            const int lx = lane + 32 * (i & 1), ly = warp + 8 * (i >> 1);
+            if (!inside(lx, ly)) continue;
+            const int x = tx0 + lx, y = ty0 + ly, q = ly * nx + lx;
+            const bool hw = INNER || x > 0, he = INNER || x + 1 < nx, hn = INNER || y > 0, hs = INNER || y + 1 < G.ny;
+            const float sv = MODE == 0 ? sva[i % kAhead] : sT[q];
+            const float ov = MODE == 0 ? ova[i % kAhead] : (rhs ? 0.f : float(oT[q]));
+            const float bc = rhs ? sv : af * (sv - ov);
+            if (MODE == 0) {
+                // ||b||^2 with b = alpha s + L o, for the relative-residual denominator
+                float bv = bc;
+                if (!rhs) {
+                    float lo = 0.f;
+                    if (hw) lo += ov - float(oT[q - 1]);
+                    if (he) lo += ov - float(oT[q + 1]);
+                    if (hn) lo += ov - float(oT[q - nx]);
+                    if (hs) lo += ov - float(oT[q + nx]);
+                    bv = fmaf(af, sv, lo);
+                }
+                bbf = fmaf(bv, bv, bbf);
+            }
+            TV rv;
+            if constexpr (MODE == 0) {
+                rv = cvt<TV>(bc);
+            } else {
+                const TS c = dsm[ly + 1][lx + 1];
+                const int deg = INNER ? 4 : int(hw) + int(he) + int(hn) + int(hs);
+                // A d in TF (FP64 when mixed): the operator on the high-precision iterate, where
+                // the cancellation between alpha d + L d and the right-hand side happens.
+                // r = bc - A d.  bc = alpha (s - o) is formed in FP32, so its own rounding (~6e-8
+                // |bc|) bounds what FP64 could add here: unless kExact, A d is rounded to the
+                // V-cycle type before the subtraction (same order of error, one FP64 operation per
+                // cell less).  That caps the reachable relative residual near 6e-8 ||bc|| / ||b||;
+                // tolerances below 1e-7 select kExact.
+                const TS w = dsm[ly + 1][lx], ea = dsm[ly + 1][lx + 2], n = dsm[ly][lx + 1], so = dsm[ly + 2][lx + 1];
+                float cf;  // d rounded to FP32
+                if constexpr (SPLIT) {
+                    cf = as_split(c).hi;
+                    rv = bc - split_apply(at_degree(ad.s, deg), as_split(c), as_split(w), as_split(ea), as_split(n),
+                                          as_split(so));
+                } else {
+                    cf = cvt<float>(c);
+                    const TF nsum = (w + ea) + (n + so);
+                    const TF Ad = fma_t(at_degree(ad.v, deg), c, -nsum);
+                    if constexpr (FORM == kRounded && sizeof(TV) < sizeof(TF)) rv = bc - cvt<TV>(Ad);
+                    else rv = cvt<TV>(cvt<TF>(bc) - Ad);
+                }
+                // output: d alone in the adjoint mode, else o + d (in FP64 when TV is FP64)
+                float f;
+                if (rhs) f = cf;
+                else if constexpr (sizeof(TV) == 8) f = cvt<float>(cvt<double>(ov) + c);
+                else f = ov + cf;
+                outT[q] = f;
+            }
+            rT[ly * G.pitch0 + lx] = rv;
+            const float rf = cvt<float>(rv);
+            rrf = fmaf(rf, rf, rrf);
+        }
+    };
+    if (tx0 >= 1 && ty0 >= 1 && tx0 + kTopTX < nx && ty0 + kTopTY < G.ny) pass(std::true_type{});
+    else pass(std::false_type{});
 #pragma unroll
     for (int m = 16; m > 0; m >>= 1) {
         rrf += __shfl_xor_sync(0xffffffffu, rrf, m);
@@ -577,6 +658,12 @@ struct Blob {
 // 1.2 M 277 / 375, 4.7 M 860 / 770.
 template <class TV>
 constexpr double kTileMaxCellsOf = sizeof(TV) == 4 ? 5e6 : 2.5e6;
+
+// Batches of at least so many cells form A d of the correction passes in split form (k_top).  Below,
+// the pass is some 5 % of a solve that latency bounds (8.4 M cells: 88 us in FP64, 70 split, in a
+// solve of 1.4 ms), and FP64 keeps the residual's last bits, which a fit that differentiates
+// differences of neighbouring slices amplifies.
+constexpr double kSplitCells = 1.6e7;
 
 template <class TF, class TV>
 struct Solver {
@@ -1071,21 +1158,31 @@ struct Solver {
         const double in_b = rq->rhs ? 4.0 : 4.0 + sizeof(To);
         const double it_b = MODE == 0 ? 0.0 : sizeof(TV) + sizeof(TF) + 4.0 + (MODE == 2 ? sizeof(TF) : 0.0);
         const double bytes = top_cells * (in_b + it_b + sizeof(TV));
-        // FP64 work of the pass (when the iterate is FP64): the 5-point operator on d, three
-        // adds and one fma per cell, plus the update d_old + e in MODE 2
-        const double flops = sizeof(TF) == 8 && MODE > 0 ? top_cells * (MODE == 2 ? 6.0 : 5.0) : 0.0;
+        // FP64 work of the pass where it bounds it (FP64 iterate, not split): the 5-point operator
+        // on d, three adds and one fma per cell, plus the update d_old + e in MODE 2
+        const bool mixed = sizeof(TV) < sizeof(TF);
+        const int form = MODE == 0 || !mixed ? kRounded
+                                             : (rq->opts.tol < 1e-7 ? kExact : (top_cells >= kSplitCells ? kSplit : kRounded));
+        const double flops = sizeof(TF) == 8 && MODE > 0 && form != kSplit ? top_cells * (MODE == 2 ? 6.0 : 5.0) : 0.0;
         KernelScope ks(MODE == 0 ? "residual_first" : "residual_update", st, bytes, flops);
         AlphaDeg<TF> ad;
-        for (int q = 0; q < 5; ++q) ad.v[q] = TF(rq->alpha) + TF(q);
+        for (int q = 0; q < 5; ++q) {
+            ad.v[q] = TF(rq->alpha) + TF(q);
+            ad.s[q].hi = float(ad.v[q]);
+            ad.s[q].lo = float(double(ad.v[q]) - double(ad.s[q].hi));
+        }
         ad.alpha_f = float(rq->alpha);
-        if (rq->opts.tol < 1e-7)
-            k_top<TF, TV, To, MODE, true><<<(unsigned)top_tiles, 256, 0, st>>>(
-                d_top, d_top_ts, (int)rq->nslices, d_active, d_call, d_state, dbuf[0], dbuf[1], rq->alpha, ad,
-                d_norms);
-        else
-            k_top<TF, TV, To, MODE, false><<<(unsigned)top_tiles, 256, 0, st>>>(
-                d_top, d_top_ts, (int)rq->nslices, d_active, d_call, d_state, dbuf[0], dbuf[1], rq->alpha, ad,
-                d_norms);
+        auto launch = [&](auto form_tag) {
+            k_top<TF, TV, To, MODE, decltype(form_tag)::value><<<(unsigned)top_tiles, 256, 0, st>>>(
+                d_top, d_top_ts, (int)rq->nslices, d_active, d_call, d_state, dbuf[0], dbuf[1], ad, d_norms);
+        };
+        if constexpr (MODE > 0 && sizeof(TV) < sizeof(TF)) {
+            if (form == kExact) launch(std::integral_constant<int, kExact>{});
+            else if (form == kSplit) launch(std::integral_constant<int, kSplit>{});
+            else launch(std::integral_constant<int, kRounded>{});
+        } else {
+            launch(std::integral_constant<int, kRounded>{});
+        }
         EMF_CHECK_LAUNCH();
         return EMFUSE_OK;
     }
