@@ -16,7 +16,7 @@ CSRC = os.path.join(PKG, "csrc")
 ROOT = os.path.dirname(PKG)
 BUILD_DIR = os.path.join(ROOT, "_build")
 LIB_PATH = os.path.join(PKG, "libemfuse.so")
-SOURCES = ["api.cu", "smooth.cu", "multigrid.cu", "fused_f32.cu", "fused_f64.cu", "fused_f32_s68.cu",
+SOURCES = ["api.cu", "smooth.cu", "smooth_packed.cu", "multigrid.cu", "fused_f32.cu", "fused_f64.cu", "fused_f32_s68.cu",
            "fused_f64_s68.cu", "tile_f32.cu", "tile_f64.cu", "runtime.cu", "dct_solve.cu", "mg3d.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2",

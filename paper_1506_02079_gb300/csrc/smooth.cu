@@ -9,7 +9,7 @@
 //     zero-fills the halo outside the stack.  x blur in items of 8 outputs, one barrier per
 //     plane, y blur of 2 x 2 outputs per thread, then a 19-plane register ring along z (moved
 //     once per block of planes, so the march stays a small rolled loop).  Needs rows whose
-//     byte pitch is a multiple of 16.
+//     byte pitch is a multiple of 16; others are packed to such a pitch first.
 //   * smooth_fused_kernel: the same data flow with plain loads, for any pitch.
 //     Each input plane is staged in shared memory with its xy halo, blurred in x then y,
 //     and pushed into a per-thread ring of the last P planes held in registers; the z-blur of
@@ -25,57 +25,19 @@
 #include <cmath>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "emfuse_common.cuh"
 #include "emfuse_internal.cuh"
+#include "smooth_tma.cuh"
 #include "tma.cuh"
 
 namespace emfuse {
 
 namespace {
 
-constexpr int kTX = 64;   // tile width (outputs)
-constexpr int kTY = 16;   // tile height (outputs)
-constexpr int kThreads = 256;
-constexpr int kMaxRxy = 8;
-
-struct SmoothParams {
-    float wxy[2 * kMaxRxy + 1];  // taps w(d), d = -Rxy..Rxy
-    float wz[19];                // wz[j] = w(Rz - j), j = 0..2Rz (zero beyond)
-    int Rxy, Rz;
-    float kappa2;                // robust averaging: squared threshold in standard deviations
-};
-
-// Robust z-average of one voxel (Sec. 3, the outlier example: only values within kappa
-// weighted standard deviations of the window's weighted mean are averaged).  v[j] are the
-// xy-smoothed window values, w[j] their tap weights (0 for taps outside the stack).
-template <int P>
-__device__ __forceinline__ float robust_window(const float (&v)[P], const float (&w)[P], float kappa2) {
-    float W = 0.f, m = 0.f;
-#pragma unroll
-    for (int j = 0; j < P; ++j) {
-        W += w[j];
-        m = fmaf(w[j], v[j], m);
-    }
-    const float mu = m / W;
-    float s2 = 0.f;
-#pragma unroll
-    for (int j = 0; j < P; ++j) {
-        const float dv = v[j] - mu;
-        s2 = fmaf(w[j] * dv, dv, s2);
-    }
-    const float thr = kappa2 * (s2 / W);
-    float sk = 0.f, wk = 0.f;
-#pragma unroll
-    for (int j = 0; j < P; ++j) {
-        const float dv = v[j] - mu;
-        const float wj = dv * dv <= thr ? w[j] : 0.f;
-        wk += wj;
-        sk = fmaf(wj, v[j], sk);
-    }
-    return sk / wk;
-}
+using namespace smooth_detail;
 
 template <class Tin>
 __device__ __forceinline__ float load_in(const Tin* p) { return float(*p); }
@@ -188,264 +150,31 @@ smooth_fused_kernel(const Tin* __restrict__ in, float* __restrict__ out, int nx,
     }
 }
 
-// ---------------------------------------------------------------- TMA-staged kernel
-// Shared-memory layout of the TMA kernel for input type Tin and xy radius R.
-template <class Tin, int R>
-struct SmTile {
-    static constexpr int HX = sizeof(Tin) == 1 ? 16 : 4;   // staged columns left of the tile: the
-                                                          // copy's x-start stays 16-byte aligned
-    static constexpr int HXR = sizeof(Tin) == 1 ? 16 : 8;  // right: a float row of 76 words is
-                                                          // 304 B, so 8 consecutive rows start in
-                                                          // 8 different 16-B bank groups
-    static constexpr int BX = kTX + HX + HXR;
-    static constexpr int BY = kTY + 2 * R;
-    static constexpr int kPlaneBytes = BX * BY * (int)sizeof(Tin);
-    static constexpr int kPlaneStride = (kPlaneBytes + 127) / 128 * 128;  // TMA destinations 128-B aligned
-    // plane buffers, all in flight except the one being blurred (about 64 KiB of copies in
-    // flight per SM with two CTAs per SM for float input)
-    static constexpr int NBUF = sizeof(Tin) == 1 ? 8 : 5;
-    static constexpr int SXW = kTX + 4;                    // x-blurred row stride (words): 272 B,
-                                                          // 8 rows -> 8 different bank groups
-    static constexpr int kRowBlocks = (BY + 7) / 8;        // x-blur items: 8 rows x 8 groups each
-    static constexpr int kXItems = 64 * kRowBlocks;        // <= 256 for R <= 4
-    static constexpr int kSmemBytes = NBUF * kPlaneStride + 2 * BY * SXW * 4 + NBUF * 8;
-};
+// Largest packed slab (see smooth_stack).
+constexpr int64_t kPackBytes = (int64_t)1 << 29;
 
-// 16 consecutive staged values (as float) starting at p.
-template <class Tin>
-__device__ __forceinline__ void load16(const Tin* p, float (&s)[16]);
-template <>
-__device__ __forceinline__ void load16<float>(const float* p, float (&s)[16]) {
+// Rows y0 .. y0 + ny_slab - 1 of planes z0 .. of `in` (any pitch) to rows of `ppitch` elements, one
+// block per row; the padding is not written (TMA reads only nx elements of a row).
+template <class T>
+__global__ void __launch_bounds__(256)
+k_pack(const T* __restrict__ in, T* __restrict__ out, int nx, int y0, int ny_slab, int64_t ny, int64_t z0, int64_t pitch,
+       int64_t ppitch, int64_t rows) {
+    for (int64_t row = blockIdx.x; row < rows; row += gridDim.x) {
+        const int64_t z = row / ny_slab, y = row - z * ny_slab;
+        const T* src = in + ((z0 + z) * ny + y0 + y) * pitch;
+        T* dst = out + row * ppitch;
+        if (sizeof(T) == 1) {  // 4 bytes per store; the last store stays inside the padded row
+            for (int x = 4 * threadIdx.x; x < nx; x += 4 * blockDim.x) {
+                uint32_t v = 0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const float4 q = reinterpret_cast<const float4*>(p)[k];
-        s[4 * k] = q.x; s[4 * k + 1] = q.y; s[4 * k + 2] = q.z; s[4 * k + 3] = q.w;
-    }
-}
-template <>
-__device__ __forceinline__ void load16<uint8_t>(const uint8_t* p, float (&s)[16]) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const uchar4 q = reinterpret_cast<const uchar4*>(p)[k];
-        s[4 * k] = q.x; s[4 * k + 1] = q.y; s[4 * k + 2] = q.z; s[4 * k + 3] = q.w;
-    }
-}
-
-// One HBM pass of the separable smoothing.  A CTA owns a 64 x 16 xy-tile and marches along z.
-// Per input plane (arriving by TMA into a ring of NBUF shared-memory buffers, zero-filled
-// outside the stack):
-//   x blur   items of 8 outputs on one staged row (rows tile + y halo), written to one of two
-//            x-blurred planes; 8 consecutive lanes take 8 rows, so the vector loads and
-//            stores of a quarter-warp fall in distinct banks;
-//   barrier  the only one per plane: the x-blurred plane is complete, the staged buffer is
-//            free and is refilled with the plane NBUF ahead;
-//   y blur   each thread 2 columns x 2 rows into a register ring of the last 19 planes;
-//   z blur   the plane Rz behind is emitted from the ring, scaled by the product of the three
-//            inverse normalisers.
-// The taps are kernel parameters with compile-time indices, i.e. constant-bank operands of the
-// FMAs.  The blurs sum in their own order and scale once at the end, so results agree with the
-// other implementations to rounding.
-template <class Tin, int R, bool ROB>
-__global__ void __launch_bounds__(kThreads, 2)
-smooth_tma_kernel(const __grid_constant__ CUtensorMap map, float* __restrict__ out, int nx, int ny, int nz,
-                  int64_t pitch, int z0, int z1, const float* __restrict__ inv_nx,
-                  const float* __restrict__ inv_ny, const float* __restrict__ inv_nz, SmoothParams prm,
-                  int* __restrict__ err) {
-    using G = SmTile<Tin, R>;
-    constexpr int P = 19;  // z taps: supports floor(3 sigma_z) <= 9
-    constexpr int NB = G::NBUF;
-    extern __shared__ __align__(128) unsigned char smem[];
-    unsigned char* s_raw = smem;
-    float* s_x = reinterpret_cast<float*>(smem + NB * G::kPlaneStride);  // [2][BY][SXW]
-    uint64_t* s_bar = reinterpret_cast<uint64_t*>(smem + NB * G::kPlaneStride + 2 * G::BY * G::SXW * 4);
-    const int tid = threadIdx.x;
-    const int x0 = blockIdx.x * kTX, y0 = blockIdx.y * kTY;
-    const int Rz = prm.Rz;
-    const int zin_lo = max(0, z0 - Rz), zin_hi = min(nz, z1 + Rz), zi_end = z1 + Rz;
-    const uint32_t bar0 = smem_addr(&s_bar[0]);
-    if (tid == 0) {
-        for (int q = 0; q < NB; ++q) mbar_init(bar0 + 8 * q, 1);
-        mbar_init_fence();
-    }
-    __syncthreads();
-    // thread 0: plane zi into buffer slot (zi - zin_lo) mod NB; a slot is refilled only after
-    // the barrier that ended the x blur of the plane it held
-    auto issue = [&](int zi, int slot) {
-        fence_proxy_async();
-        mbar_expect_tx(bar0 + 8 * slot, G::kPlaneBytes);
-        tma_load_3d(smem_addr(s_raw + slot * G::kPlaneStride), &map, x0 - G::HX, y0 - R, zi, bar0 + 8 * slot);
-    };
-    if (tid == 0)
-        for (int q = 0; q < NB && zin_lo + q < zin_hi; ++q) issue(zin_lo + q, q);
-
-    // x-blur item of this thread (warp-uniform participation: kXItems is a multiple of 64)
-    const bool xw = tid < G::kXItems;
-    const int xr = (tid >> 6) * 8 + (tid & 7);  // staged row
-    const int xg = (tid >> 3) & 7;              // group of 8 output columns
-    const bool xitem = xw && xr < G::BY;
-    const Tin* const s_in0 = reinterpret_cast<const Tin*>(s_raw) + xr * G::BX + 8 * xg + G::HX - 4;
-    float* const sx_item = s_x + xr * G::SXW + 8 * xg;
-    // y/z outputs of this thread: columns 2 lane, 2 lane + 1 of rows 2 warp, 2 warp + 1
-    const int lane = tid & 31, wrp = tid >> 5;
-    const int gx = x0 + 2 * lane;
-    const int gy0 = y0 + 2 * wrp, gy1 = gy0 + 1;
-    const float* const sy_col = s_x + (2 * wrp) * G::SXW + 2 * lane;
-    float sxy[4];  // inv_x * inv_y of the 4 outputs (row 0 x, row 0 x+1, row 1 x, row 1 x+1)
-    {
-        const float ix0 = inv_nx[min(gx, nx - 1)], ix1 = inv_nx[min(gx + 1, nx - 1)];
-        const float iy0 = inv_ny[min(gy0, ny - 1)], iy1 = inv_ny[min(gy1, ny - 1)];
-        sxy[0] = ix0 * iy0; sxy[1] = ix1 * iy0; sxy[2] = ix0 * iy1; sxy[3] = ix1 * iy1;
-    }
-    const bool st0 = gy0 < ny, st1 = gy1 < ny;
-    const bool vec2 = (pitch & 1) == 0 && (reinterpret_cast<uintptr_t>(out) & 7) == 0 && gx + 1 < nx;
-    float* const dst0 = out + (int64_t)min(gy0, ny - 1) * pitch + gx;
-    float* const dst1 = out + (int64_t)min(gy1, ny - 1) * pitch + gx;
-
-    // z ring: slots 0 .. P-2 hold the P-1 planes before the current block of U planes, slots
-    // P-1 .. P-2+U the block; the ring moves by U slots once per block (the loop over a block is
-    // unrolled, so every slot index is a constant)
-    constexpr int U = ROB ? 2 : 4;  // the robust window needs more registers of its own
-    float ring[P - 1 + U][4];
-#pragma unroll
-    for (int q = 0; q < P - 1 + U; ++q)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) ring[q][c] = 0.f;
-    const int64_t plane = pitch * (int64_t)ny;
-
-    int slot = 0;        // buffer slot of plane zi
-    uint32_t phase = 0;  // barrier parity of the current lap over the slots
-    int buf = 0;         // x-blurred plane buffer (0 or 1)
-#pragma unroll 1
-    for (int zb = zin_lo; zb < zi_end; zb += U) {
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int zi = zb + u;
-            float v[4] = {0.f, 0.f, 0.f, 0.f};
-            if (zi < zin_hi) {  // uniform across the CTA
-                bool ok = true;
-                const int boff = buf * (G::BY * G::SXW);
-                if (xw) {
-                    ok = mbar_wait_warp(bar0 + 8 * slot, phase);
-                    if (ok && xitem) {
-                        float s[16];
-                        load16<Tin>(s_in0 + slot * (G::kPlaneStride / (int)sizeof(Tin)), s);
-                        // output i sits at s[4 + i]
-                        float o[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            float acc = prm.wxy[0] * s[4 + i - R];
-#pragma unroll
-                            for (int d = -R + 1; d <= R; ++d) acc = fmaf(prm.wxy[d + R], s[4 + i + d], acc);
-                            o[i] = acc;
-                        }
-                        float4* dst = reinterpret_cast<float4*>(sx_item + boff);
-                        dst[0] = make_float4(o[0], o[1], o[2], o[3]);
-                        dst[1] = make_float4(o[4], o[5], o[6], o[7]);
-                    }
-                }
-                if (!__syncthreads_and(ok)) {
-                    // give up: flag the host, let the copies in flight land, leave
-                    if (tid == 0) {
-                        atomicExch(err, 1);
-                        for (int zz = zi; zz < zin_hi && zz < zi + NB; ++zz) {
-                            const int k = zz - zin_lo;
-                            const uint32_t b = bar0 + 8 * (k % NB), ph = (uint32_t)((k / NB) & 1);
-                            for (int it = 0; it < kWaitLimit; ++it)
-                                if (mbar_try_wait(b, ph)) break;
-                        }
-                    }
-                    __syncthreads();
-                    return;
-                }
-                if (tid == 0 && zi + NB < zin_hi) issue(zi + NB, slot);
-                // y blur of rows 2 warp, 2 warp + 1 (x-blurred rows 2 warp .. 2 warp + 2R + 1)
-#pragma unroll
-                for (int t = 0; t <= 2 * R + 1; ++t) {
-                    const float2 q = *reinterpret_cast<const float2*>(sy_col + boff + t * G::SXW);
-                    if (t == 0) {
-                        v[0] = prm.wxy[0] * q.x;
-                        v[1] = prm.wxy[0] * q.y;
-                    } else if (t <= 2 * R) {
-                        v[0] = fmaf(prm.wxy[t], q.x, v[0]);
-                        v[1] = fmaf(prm.wxy[t], q.y, v[1]);
-                    }
-                    if (t == 1) {
-                        v[2] = prm.wxy[0] * q.x;
-                        v[3] = prm.wxy[0] * q.y;
-                    } else if (t >= 2) {
-                        v[2] = fmaf(prm.wxy[t - 1], q.x, v[2]);
-                        v[3] = fmaf(prm.wxy[t - 1], q.y, v[3]);
-                    }
-                }
-                if (R == 0) {  // 2R + 1 = 1 row per output
-                    const float2 q = *reinterpret_cast<const float2*>(sy_col + boff + G::SXW);
-                    v[2] = prm.wxy[0] * q.x;
-                    v[3] = prm.wxy[0] * q.y;
-                }
-                if (++slot == NB) { slot = 0; phase ^= 1u; }
-                buf ^= 1;
+                for (int i = 0; i < 4; ++i)
+                    if (x + i < nx) v |= (uint32_t)(uint8_t)src[x + i] << (8 * i);
+                *reinterpret_cast<uint32_t*>(dst + x) = v;
             }
-#pragma unroll
-            for (int c = 0; c < 4; ++c) ring[P - 1 + u][c] = v[c];
-            // emit plane zi - Rz from ring slots u .. u + P - 1 (slot u + P - 1 = plane zi)
-            const int zo = zi - Rz;
-            if (zo >= z0 && zo < z1) {  // uniform across the CTA
-                float o[4];
-                if constexpr (ROB) {
-                    float wv[P];
-#pragma unroll
-                    for (int jj = 0; jj < P; ++jj) wv[jj] = (zi - jj >= 0 && zi - jj < nz) ? prm.wz[jj] : 0.f;
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        float vv[P];
-#pragma unroll
-                        for (int jj = 0; jj < P; ++jj) vv[jj] = ring[u + P - 1 - jj][c];
-                        o[c] = robust_window<P>(vv, wv, prm.kappa2) * sxy[c];
-                    }
-                } else {
-                    const float inz = inv_nz[zo];
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        float acc = prm.wz[0] * ring[u + P - 1][c];
-#pragma unroll
-                        for (int jj = 1; jj < P; ++jj) acc = fmaf(prm.wz[jj], ring[u + P - 1 - jj][c], acc);
-                        o[c] = acc * (sxy[c] * inz);
-                    }
-                }
-                const int64_t zoff = (int64_t)(zo - z0) * plane;
-                if (vec2) {
-                    if (st0) *reinterpret_cast<float2*>(dst0 + zoff) = make_float2(o[0], o[1]);
-                    if (st1) *reinterpret_cast<float2*>(dst1 + zoff) = make_float2(o[2], o[3]);
-                } else {
-                    if (st0 && gx < nx) dst0[zoff] = o[0];
-                    if (st0 && gx + 1 < nx) dst0[zoff + 1] = o[1];
-                    if (st1 && gx < nx) dst1[zoff] = o[2];
-                    if (st1 && gx + 1 < nx) dst1[zoff + 1] = o[3];
-                }
-            }
+        } else {
+            for (int x = threadIdx.x; x < nx; x += blockDim.x) dst[x] = src[x];
         }
-#pragma unroll
-        for (int q = 0; q < P - 1; ++q)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) ring[q][c] = ring[q + U][c];
     }
-}
-
-// Opt in to the TMA kernel's dynamic shared memory once per instantiation and device.
-template <class Tin, int R, bool ROB>
-int smooth_tma_prepare() {
-    static std::mutex mu;
-    static bool done[64] = {false};
-    int dev = 0;
-    EMF_CUDA(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return EMFUSE_OK;
-    std::lock_guard<std::mutex> lk(mu);
-    if (!done[dev]) {
-        EMF_CUDA(cudaFuncSetAttribute(smooth_tma_kernel<Tin, R, ROB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      SmTile<Tin, R>::kSmemBytes));
-        done[dev] = true;
-    }
-    return EMFUSE_OK;
 }
 
 struct AxisParams {
@@ -569,58 +298,94 @@ int smooth_stack(const void* in, int dt, float* out, int64_t nx, int64_t ny, int
     const float* inv_z = inv_y + ny;
 
     const size_t esz = dt == EMFUSE_U8 ? 1 : 4;
-    const bool tma_ok = Rxy <= 4 && Rz <= 9 && force_path == 0 && (pitch * (int64_t)esz) % 16 == 0 &&
-                        (reinterpret_cast<uintptr_t>(in) & 15) == 0;
-    if (tma_ok) {
-        SmoothParams prm{};
-        prm.Rxy = Rxy;
-        prm.Rz = Rz;
-        for (int d = 0; d < 2 * Rxy + 1; ++d) prm.wxy[d] = wxy[d];
-        for (int j = 0; j < 2 * Rz + 1; ++j) prm.wz[j] = wz[2 * Rz - j];
-        prm.kappa2 = kappa * kappa;
-        CUtensorMap map;
+    const bool tma_ok = Rxy <= 4 && Rz <= 9 && force_path == 0;
+    const bool aligned = (pitch * (int64_t)esz) % 16 == 0 && (reinterpret_cast<uintptr_t>(in) & 15) == 0;
+    if (tma_ok && (aligned || (Rxy >= 1 && Rz >= 1))) {
+        SmoothTmaCall c{};
+        c.prm.Rxy = Rxy;
+        c.prm.Rz = Rz;
+        for (int d = 0; d < 2 * Rxy + 1; ++d) c.prm.wxy[d] = wxy[d];
+        for (int j = 0; j < 2 * Rz + 1; ++j) c.prm.wz[j] = wz[2 * Rz - j];
+        c.prm.kappa2 = kappa * kappa;
+        c.out = out;
+        c.nx = (int)nx;
+        c.ny = (int)ny;
+        c.nz = (int)nz;
+        c.pitch = pitch;
+        c.z0 = (int)z0;
+        c.z1 = (int)z1;
+        c.inv_x = inv_x;
+        c.inv_y = inv_y;
+        c.inv_z = inv_z;
+        c.yend = (int)ny;
+        c.err = device_error_flag();
         const int hx = dt == EMFUSE_U8 ? 16 : 4, hxr = dt == EMFUSE_U8 ? 16 : 8;
-        EMF_TRY(encode_tensor_map_3d(&map, in, (int)esz, nx, ny, nz, pitch, kTX + hx + hxr, kTY + 2 * Rxy));
-        int* err = device_error_flag();
-        if (!err) {
+        if (!c.err) {
             set_error("could not allocate the device error word");
             return EMFUSE_ECUDA;
         }
-        dim3 grid((unsigned)ceil_div(nx, kTX), (unsigned)ceil_div(ny, kTY));
         const int64_t zin0 = std::max<int64_t>(0, z0 - Rz), zin1 = std::min<int64_t>(nz, z1 + Rz);
-        {
-            KernelScope ks(rob ? "smooth_tma_robust" : "smooth_tma", st,
-                           (double)nx * ny * ((zin1 - zin0) * (double)esz + (z1 - z0) * 4.0));
-#define EMF_SMOOTH_TMA2(TT, RR, RB)                                                                \
-    do {                                                                                           \
-        EMF_TRY((smooth_tma_prepare<TT, RR, RB>()));                                               \
-        smooth_tma_kernel<TT, RR, RB><<<grid, kThreads, SmTile<TT, RR>::kSmemBytes, st>>>(          \
-            map, out, (int)nx, (int)ny, (int)nz, pitch, (int)z0, (int)z1, inv_x, inv_y, inv_z, prm, err);       \
-    } while (0)
-#define EMF_SMOOTH_TMA1(RR, RB)                                                                    \
-    do {                                                                                           \
-        if (dt == EMFUSE_U8) EMF_SMOOTH_TMA2(uint8_t, RR, RB);                                     \
-        else EMF_SMOOTH_TMA2(float, RR, RB);                                                       \
-    } while (0)
-#define EMF_SMOOTH_TMA(RR)                                                                         \
-    do {                                                                                           \
-        if (rob) EMF_SMOOTH_TMA1(RR, true);                                                        \
-        else EMF_SMOOTH_TMA1(RR, false);                                                           \
-    } while (0)
+        const double bytes = (double)nx * ((zin1 - zin0) * (double)esz + (z1 - z0) * 4.0);  // per row
+        if (aligned) {
+            EMF_TRY(encode_tensor_map_3d(&c.map, in, (int)esz, nx, ny, nz, pitch, kTX + hx + hxr, kTY + 2 * Rxy));
+            KernelScope ks(rob ? "smooth_tma_robust" : "smooth_tma", st, bytes * ny);
+            auto run = [&](auto radius) -> int {
+                constexpr int R = decltype(radius)::value;
+                if (dt == EMFUSE_U8)
+                    return rob ? smooth_tma_launch<uint8_t, R, true, false, 19>(c, st)
+                               : smooth_tma_launch<uint8_t, R, false, false, 19>(c, st);
+                return rob ? smooth_tma_launch<float, R, true, false, 19>(c, st)
+                           : smooth_tma_launch<float, R, false, false, 19>(c, st);
+            };
             switch (Rxy) {
-                case 0: EMF_SMOOTH_TMA(0); break;
-                case 1: EMF_SMOOTH_TMA(1); break;
-                case 2: EMF_SMOOTH_TMA(2); break;
-                case 3: EMF_SMOOTH_TMA(3); break;
-                default: EMF_SMOOTH_TMA(4); break;
+                case 0: return run(std::integral_constant<int, 0>{});
+                case 1: return run(std::integral_constant<int, 1>{});
+                case 2: return run(std::integral_constant<int, 2>{});
+                case 3: return run(std::integral_constant<int, 3>{});
+                default: return run(std::integral_constant<int, 4>{});
             }
-#undef EMF_SMOOTH_TMA
-#undef EMF_SMOOTH_TMA1
-#undef EMF_SMOOTH_TMA2
-            EMF_CHECK_LAUNCH();
+            // a timed-out wait is reported by the next call that synchronises (the solves)
         }
-        // a timed-out wait is reported by the next call that synchronises (the solves)
-        return EMFUSE_OK;
+        // Rows that TMA cannot read (a byte pitch or base that is no multiple of 16): slabs of rows
+        // of the needed planes, with their halo rows, are copied to an aligned pitch first.  The
+        // copy costs 2 (uint8) or 8 bytes per voxel: 32 x 2047 x 2049 uint8 0.10 ms and the kernel 0.44
+        // where smooth_fused_kernel took 2.32 (float 0.29 and 0.45 for 2.52; robust 1.68 for 3.73
+        // and 1.95 for 4.06, copy included).  A slab is at most kPackBytes; where not even one
+        // tile's rows fit, or there is no memory for it, smooth_fused_kernel still runs.
+        const int64_t ppitch = round_up(nx, 16 / (int64_t)esz), nzin = zin1 - zin0;
+        const int64_t row_bytes = nzin * ppitch * (int64_t)esz;
+        int64_t rows = std::min<int64_t>(ny, kPackBytes / row_bytes - 2 * Rxy);  // output rows of a slab
+        if (rows < ny) rows = rows / kTY * kTY;
+        DeviceBuffer slab;
+        if (rows >= 1 && slab.alloc((size_t)(std::min<int64_t>(ny, rows + 2 * Rxy) * row_bytes), st) == EMFUSE_OK) {
+            for (int64_t ya = 0; ya < ny; ya += rows) {
+                const int64_t yb = std::min(ny, ya + rows);
+                const int64_t ra = std::max<int64_t>(0, ya - Rxy), rb = std::min<int64_t>(ny, yb + Rxy);
+                {
+                    KernelScope ks("smooth_pack", st, (double)(2 * esz) * nx * (rb - ra) * nzin);
+                    const int64_t n = nzin * (rb - ra);
+                    const unsigned grid = (unsigned)std::min<int64_t>(n, (int64_t)kNumSMs * 32);
+                    if (dt == EMFUSE_U8)
+                        k_pack<uint8_t><<<grid, 256, 0, st>>>((const uint8_t*)in, slab.as<uint8_t>(), (int)nx, (int)ra,
+                                                              (int)(rb - ra), ny, zin0, pitch, ppitch, n);
+                    else
+                        k_pack<float><<<grid, 256, 0, st>>>((const float*)in, slab.as<float>(), (int)nx, (int)ra,
+                                                            (int)(rb - ra), ny, zin0, pitch, ppitch, n);
+                    EMF_CHECK_LAUNCH();
+                }
+                EMF_TRY(encode_tensor_map_3d(&c.map, slab.as<char>(), (int)esz, nx, rb - ra, nzin, ppitch, kTX + hx + hxr,
+                                             kTY + 2 * Rxy));
+                c.ybase = (int)ya;
+                c.yend = (int)yb;
+                c.ymap = (int)ra;
+                c.zmap = (int)zin0;
+                KernelScope ks(rob ? "smooth_packed_robust" : "smooth_packed", st, bytes * (yb - ya));
+                EMF_TRY(smooth_tma_packed(c, dt, rob, st));
+            }
+            return EMFUSE_OK;
+        }
+        cudaGetLastError();  // no memory for the copy: not an error of this call
+        set_error("");
     }
     const bool fused_ok = Rxy <= kMaxRxy && Rz <= 9 && force_path != 1;
     if (fused_ok) {
