@@ -7,6 +7,8 @@
 #include <mutex>
 
 #include "fused_impl.cuh"
+#include "tail_cells.cuh"
+#include "tail_warps.cuh"
 
 namespace emfuse {
 namespace fused_detail {
@@ -91,20 +93,25 @@ int launch_wave_impl(const WaveArgs<T>& a, int S, bool zero_init, bool up, cudaS
 template <class T>
 int launch_tail_impl(const TailArgs<T>& a, cudaStream_t st, double bytes) {
     if (a.nslices == 0) return EMFUSE_OK;
+    constexpr bool warps = sizeof(T) == 4;  // tail_warps.cuh says why
+    constexpr int smem = warps ? (int)sizeof(fused_detail::TailShared<T>) : fused_detail::cells_smem_bytes<T>();
+    auto* kernel = [] {
+        if constexpr (warps) return fused_detail::k_tail<T>;
+        else return fused_detail::k_tail_cells<T>;
+    }();
     static std::mutex mu;
-    static int attr_set[64] = {0};  // the shared-memory limit set per device
+    static bool done[64] = {false};
     int dev = 0;
     EMF_CUDA(cudaGetDevice(&dev));
     if (dev >= 0 && dev < 64) {
         std::lock_guard<std::mutex> lk(mu);
-        if (attr_set[dev] < a.smem_bytes) {
-            EMF_CUDA(cudaFuncSetAttribute(fused_detail::k_tail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          a.smem_bytes));
-            attr_set[dev] = a.smem_bytes;
+        if (!done[dev]) {
+            EMF_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+            done[dev] = true;
         }
     }
     KernelScope ks("coarse_tail", st, bytes);
-    fused_detail::k_tail<T><<<(unsigned)a.nslices, fused_detail::kTailThreads, (size_t)a.smem_bytes, st>>>(a);
+    kernel<<<(unsigned)a.nslices, fused_detail::kTailThreads, smem, st>>>(a);
     EMF_CHECK_LAUNCH();
     return EMFUSE_OK;
 }

@@ -47,8 +47,7 @@ __device__ __forceinline__ Coef<T> tile_coef(const TailCoef<T>* tab, int x, int 
     return tail_coef<T>(tab + 4 * tail_class(y, ny) + tail_class(x, nx));
 }
 
-// Stencils of a column on inner rows (iD, D) and on a full first or last row (iDb, Db), where
-// one face less enters the diagonal; all 0 outside the level.
+// Stencils of a column (col_stencil), split for vector loads.
 template <class T>
 struct alignas(16) ColCoef {
     T cw, ce, cy, iD;
@@ -57,9 +56,6 @@ template <class T>
 struct ColDiag {
     T iDb, D, Db;
 };
-
-// Rows of a tile: inner, first / last with full cells, outside the level, of partial cells.
-enum : unsigned char { kRowInner = 0, kRowEdge = 1, kRowOut = 2, kRowPartial = 3 };
 
 template <class T, bool ZERO, bool UP>
 __global__ void __launch_bounds__(TileShape<T>::kWarps * 32, 2) k_tile(TileArgs<T> a) {
@@ -85,46 +81,29 @@ __global__ void __launch_bounds__(TileShape<T>::kWarps * 32, 2) k_tile(TileArgs<
     // stencils and interpolation weights of the tile's columns and rows, one per thread
     if (tid < kWaveWidth) {
         const int xc = X0 - a.hx + tid, q = tid & 3, l = tid >> 2;
-        ColCoef<T> c{T(0), T(0), T(0), T(0)};
-        ColDiag<T> d{T(0), T(0), T(0)};
         T w = T(0);
-        if (xc >= 0 && xc < nx) {
-            const AxisCoef<T> ax = axis_coef<T>(xc, nx, L.n0x, k);
-            AxisCoef<T> ay;
-            ay.w = T(1); ay.gm = T(1); ay.gp = T(1);
-            const Coef<T> m = make_coef<T>(ax, ay, k, a.alpha, a.sk);
-            ay.gm = T(0);
-            const Coef<T> e = make_coef<T>(ax, ay, k, a.alpha, a.sk);
-            c.cw = m.cw; c.ce = m.ce; c.cy = m.cn; c.iD = m.iD;
-            d.iDb = e.iD; d.D = m.D; d.Db = e.D;
-            if (UP) {
-                int I, J;
-                interp_axis<T>(xc, L.n0x, k, L.ncx, I, J, w);
-            }
+        const ColStencil<T> st = col_stencil<T>(xc, nx, L.n0x, k, a.alpha, a.sk);
+        const ColCoef<T> c{st.cw, st.ce, st.cy, st.iD};
+        const ColDiag<T> d{st.iDb, st.D, st.Db};
+        if (UP && xc >= 0 && xc < nx) {
+            int I, J;
+            interp_axis<T>(xc, L.n0x, k, L.ncx, I, J, w);
         }
         col[q][l] = c;
         diag[q][l] = d;
         if (UP) colw[q][l] = w;
     } else if (tid < kWaveWidth + TileShape<T>::kRows) {
         const int q = tid - kWaveWidth, yr = Y0 - a.hy + q;
-        unsigned char m = kRowOut;
         T w = T(0);
-        if (yr >= 0 && yr < ny) {
-            const AxisCoef<T> ay = axis_coef<T>(yr, ny, L.n0y, k);
-            const bool n1 = ay.gm == T(1), s1 = ay.gp == T(1), n0 = ay.gm == T(0), s0 = ay.gp == T(0);
-            m = ay.w != T(1) || !(n0 || n1) || !(s0 || s1) || (n0 && s0) ? kRowPartial
-                                                                         : (n1 && s1 ? kRowInner : kRowEdge);
-            if (UP) {
-                int I, J;
-                interp_axis<T>(yr, L.n0y, k, L.ncy, I, J, w);
-            }
+        if (UP && yr >= 0 && yr < ny) {
+            int I, J;
+            interp_axis<T>(yr, L.n0y, k, L.ncy, I, J, w);
         }
-        rowm[q] = m;
+        rowm[q] = row_mode<T>(yr, ny, L.n0y, k);
         if (UP) roww[q] = w;
     } else if (tid >= TileShape<T>::kWarps * 32 - 16) {
         const int q = tid & 15;
-        auto rep = [](int cls, int n) { return cls == 0 ? 0 : (cls == 1 ? min(1, n - 1) : max(0, n - 4 + cls)); };
-        const Coef<T> c = coef_at<T>(rep(q & 3, nx), rep(q >> 2, ny), nx, ny, L.n0x, L.n0y, k, a.alpha, a.sk);
+        const Coef<T> c = coef_at<T>(tail_class_rep(q & 3, nx), tail_class_rep(q >> 2, ny), nx, ny, L.n0x, L.n0y, k, a.alpha, a.sk);
         TailCoef<T>& o = tab[q];
         o.cw = c.cw; o.ce = c.ce; o.cn = c.cn; o.cs = c.cs; o.iD = c.iD; o.D = c.D;
     }

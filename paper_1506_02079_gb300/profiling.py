@@ -67,8 +67,8 @@ _KERNEL_SOURCES = {
     "residual": ("multigrid.cu", "split.cuh", "fpconv.cuh", "mg_fused.cuh", "emfuse_common.cuh"),
     "wave": ("fused_impl.cuh", "fused_launch.cuh", "fused_f32.cu", "fused_f64.cu", "fused_f32_s68.cu",
              "fused_f64_s68.cu", "mg_fused.cuh", "tma.cuh", "emfuse_common.cuh"),
-    "coarse_tail": ("fused_impl.cuh", "fused_launch.cuh", "fused_f32.cu", "fused_f64.cu", "mg_fused.cuh",
-                    "emfuse_common.cuh"),
+    "coarse_tail": ("tail_warps.cuh", "tail_cells.cuh", "fused_impl.cuh", "fused_launch.cuh", "fused_f32.cu",
+                    "fused_f64.cu", "mg_fused.cuh", "emfuse_common.cuh"),
     "tile": ("tile_impl.cuh", "tile_f32.cu", "tile_f64.cu", "fused_impl.cuh", "mg_fused.cuh", "emfuse_common.cuh"),
     "smooth": ("smooth.cu", "smooth_tma.cuh", "smooth_packed.cu", "tma.cuh", "emfuse_common.cuh"),
 }
