@@ -657,15 +657,12 @@ int emfuse_backward(const float* grad_f, const float* f, const float* s, const v
         gs = tmp_s.as<float>();
     }
     if (gs) EMF_TRY(scale_copy(lam.as<float>(), gs, n, (float)alpha, st));
-    if (grad_o) EMF_TRY(apply_laplacian_stack(lam.as<float>(), grad_o, nx, ny, nz, 1.f, st));
+    if (grad_o) EMF_TRY(apply_laplacian_stack(lam.as<float>(), grad_o, nx, ny, nz, false, st));
     if (grad_alpha) EMF_TRY(dot_diff(lam.as<float>(), s, f, n, grad_alpha, st));
     if (grad_in0) {
         // dl/dI0 = L lam + K^T (alpha lam)
         EMF_TRY(smooth_transpose(gs, grad_in0, nx, ny, nz, sigma_xy, sigma_z, st));
-        DeviceBuffer lap;
-        EMF_TRY(lap.alloc((size_t)n * sizeof(float), st));
-        EMF_TRY(apply_laplacian_stack(lam.as<float>(), lap.as<float>(), nx, ny, nz, 1.f, st));
-        EMF_TRY(axpy(lap.as<float>(), grad_in0, n, 1.f, st));
+        EMF_TRY(apply_laplacian_stack(lam.as<float>(), grad_in0, nx, ny, nz, true, st));
     }
     if (grad_sigma_z) {
         DeviceBuffer dk;

@@ -63,6 +63,12 @@ class KernelScope {
 inline int64_t round_up(int64_t a, int64_t b) { return (a + b - 1) / b * b; }
 inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
+// a / b of non-negative indexes, in 32 bits where both fit (a 64-bit division is about 100 instructions).
+__device__ __forceinline__ int64_t index_div(int64_t a, int64_t b) {
+    if (((a | b) >> 32) == 0) return (int64_t)((uint32_t)a / (uint32_t)b);
+    return a / b;
+}
+
 constexpr int kNumSMs = 152;  // GB300: 2 dies x 76 SMs (grids are sized from the device query)
 
 // Instrumentation state (runtime.cu): whether per-launch event timing is on, and the count

@@ -70,12 +70,11 @@ int gd_multigrid(const void* in, int dt, float* out, int64_t nx, int64_t ny, int
 void release_fft_plans();  // and the cuBLAS handles
 
 // elementwise helpers used by the adjoint (multigrid.cu)
-int apply_laplacian_stack(const float* in, float* out, int64_t nx, int64_t ny, int64_t nz,
-                          float scale, cudaStream_t st);
+// out = L in, or out += L in (add)
+int apply_laplacian_stack(const float* in, float* out, int64_t nx, int64_t ny, int64_t nz, bool add, cudaStream_t st);
 // sum_j <a_j, b_j - c_j> in FP64 over a dense float stack; result copied to host
 int dot_diff(const float* a, const float* b, const float* c, int64_t n, double* host_out,
              cudaStream_t st);
 int scale_copy(const float* in, float* out, int64_t n, float a, cudaStream_t st);
-int axpy(const float* x, float* y, int64_t n, float a, cudaStream_t st);
 
 }  // namespace emfuse
