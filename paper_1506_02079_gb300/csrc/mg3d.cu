@@ -108,10 +108,12 @@ __device__ __forceinline__ Coef3 table_entry(int t, int nx, int ny, int nz, cons
 //
 // The source and destination differ: tiles read their halo while neighbours write.
 //
-// Bound by instruction issue (about 50 per cell at S = 4, halo included) at one CTA of 16 warps
-// per SM; S = 4 keeps 7 planes in registers, the right-hand sides of the planes under way are kept
-// in shared memory.  32 x 1024 x 1024: DOWN 0.25 ms, UP with the addition to d 0.53 ms; one kernel per
-// half-sweep, restriction and prolongation took 0.89 and 0.84 (and 0.11 for the addition).
+// Bound by instruction issue (about 50 per cell at S = 4, halo included; 65 % of the slots) at one CTA of
+// 16 warps per SM; S = 4 keeps 6 or 7 planes in registers.  What is on its way (iterate,
+// right-hand side, coarse plane, correction) goes to shared memory by asynchronous copies: prefetched
+// into registers it made the UP leg spill, and the correction was read where it was needed (0.53 ms).
+// 32 x 1024 x 1024: DOWN 0.25 ms, UP with the addition to d 0.36 ms; one kernel per half-sweep,
+// restriction and prolongation took 0.89 and 0.84 (and 0.11 for the addition).
 constexpr int kWarps3 = 16, kRows3 = 4, kTile3 = 64;
 
 struct Leg3 {
@@ -131,10 +133,32 @@ struct Leg3 {
     float alpha, sk;
 };
 
-template <int S>
+constexpr int kCoarse3 = kRows3 / 2 + 2, kCoarseW3 = kTile3 / 2 + 2;  // coarse rows and columns of a warp
+
+// Shared memory of a leg: right-hand sides of S + 2 (residual: S + 3) planes and two planes of the
+// iterate, the ones on their way included, edge rows of S + 2 planes, and for UP a plane of the
+// correction and the warps' rows of a coarse plane on their way.
+template <int S, bool UP>
 constexpr int leg3_smem() {
-    return (S + 2) * (kTile3 * kTile3 + kWarps3 * 2 * kTile3) * (int)sizeof(float);
+    return ((UP ? S + 6 : S + 5) * kTile3 * kTile3 + (S + 2) * kWarps3 * 2 * kTile3 +
+            (UP ? kWarps3 * kCoarse3 * kCoarseW3 : 0)) * (int)sizeof(float);
 }
+
+// 8 bytes to shared memory (the last 8 - bytes of them zeros), 4 or 16 bytes; complete after copies_done().
+__device__ __forceinline__ void copy8(float* to, const float* from, int bytes) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"((unsigned)__cvta_generic_to_shared(to)), "l"(from),
+                 "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ void copy4(float* to, const float* from) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(to)), "l"(from)
+                 : "memory");
+}
+__device__ __forceinline__ void copy16(float* to, const void* from) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(to)), "l"(from)
+                 : "memory");
+}
+__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 constexpr int kOut3 = 8;  // "missing neighbours" of a column or row outside the level
 
@@ -153,12 +177,16 @@ __device__ __noinline__ float general_sum(const Coef3* q, float b, float uw, flo
 
 template <int S, bool ZERO, bool UP>
 __global__ void __launch_bounds__(kWarps3 * 32, 1) k3_leg(const Leg3 a) {
-    constexpr int NS = S + 2;                 // planes in the rings
+    constexpr int NS = S + 2;                 // planes of edge rows
+    constexpr int NB = UP ? S + 2 : S + 3;    // planes of right-hand sides (a residual is one plane behind)
     constexpr int NP = UP ? S + 2 : S + 3;    // planes in registers: T - NP + 1 .. T
     constexpr int R = kRows3;
     extern __shared__ __align__(16) float smem3[];
-    float* const bring = smem3;                            // [NS][64][64] right-hand sides, own cells only
-    float* const edge = smem3 + NS * kTile3 * kTile3;      // [NS][warp][first, last row][64]
+    float* const bring = smem3;                            // [NB][64][64] right-hand sides, own cells only
+    float* const edge = smem3 + NB * kTile3 * kTile3;      // [NS][warp][first, last row][64]
+    float* const uplane = edge + NS * kWarps3 * 2 * kTile3;  // [2][64][64] of the iterate, own cells only
+    float* const dplane = uplane + 2 * kTile3 * kTile3;      // UP: [64][64] of the correction, own cells only
+    float* const cplane = dplane + 2 * kTile3 * kTile3;      // UP: [warp][kCoarse3][kCoarseW3]
     __shared__ Coef3 tab[64];
     // levels of full cells: 1 / D and D of a cell with c missing neighbours, 0 for cells outside
     __shared__ float itab[kOut3 + kOut3 + 3], dtab[kOut3 + kOut3 + 3];
@@ -221,85 +249,113 @@ __global__ void __launch_bounds__(kWarps3 * 32, 1) k3_leg(const Leg3 a) {
     for (int q = 0; q < NP; ++q)
 #pragma unroll
         for (int r = 0; r < R; ++r) w[q][r][0] = w[q][r][1] = 0.f;
-    float2 pu[R], pb[R];  // plane T + 1 on its way
+    // Plane T + 1 is on its way while plane T is worked on, by asynchronous copies: registers are short.
+    // Right-hand sides of cells outside the level stay 0, of planes outside are not used.
     const int64_t first_row = (int64_t)Tb * ny + y;
     const float* bsrc = a.b + first_row * a.bp + x;     // next plane to fetch, this lane's first cell
     const float* usrc = ZERO ? nullptr : a.src + first_row * a.sp + x;
     const int64_t bstep = (int64_t)ny * a.bp, ustep = (int64_t)ny * a.sp;
-    // (the padding of a row is masked when the plane is taken, not here, so that nothing waits for
-    // the loads before then)
+    float* const own = bring + row0 * kTile3 + 2 * lane;
+#pragma unroll
+    for (int q = 0; q < NB; ++q)
+#pragma unroll
+        for (int r = 0; r < R; ++r) *reinterpret_cast<float2*>(own + (q * kTile3 + r) * kTile3) = make_float2(0.f, 0.f);
+    __syncthreads();
+    int bslot = Tb % NB;         // ring slot of the next plane to fetch
     auto fetch = [&](int z) {
         const bool in = z < nz && col0;
+        float* const to = own + bslot * kTile3 * kTile3;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            pu[r] = pb[r] = make_float2(0.f, 0.f);
+            float* const ut = uplane + (((z & 1) * kTile3 + row0 + r) * kTile3 + 2 * lane);
             if (in && (rows_in >> r & 1)) {
-                pb[r] = *reinterpret_cast<const float2*>(bsrc + r * a.bp);
+                copy8(to + r * kTile3, bsrc + r * a.bp, col1 ? 8 : 4);
                 if (!ZERO) {
                     const float* p = usrc + r * a.sp;
                     if (a.svec) {
-                        pu[r] = *reinterpret_cast<const float2*>(p);
+                        copy8(ut, p, col1 ? 8 : 4);
                     } else {
-                        pu[r].x = p[0];
-                        if (col1) pu[r].y = p[1];
+                        copy4(ut, p);
+                        if (col1) copy4(ut + 1, p + 1);
+                        else ut[1] = 0.f;
                     }
                 }
+            } else if (!ZERO) {
+                *reinterpret_cast<float2*>(ut) = make_float2(0.f, 0.f);
             }
         }
+        bslot = bslot + 1 == NB ? 0 : bslot + 1;
         bsrc += bstep;
         if (!ZERO) usrc += ustep;
     };
     fetch(Tb);
     // UP: coarse planes zp = (T - 1) / 2 (rounded down) in h0 and zp + 1 in h1, interpolated along x at
-    // the lane's two columns, rows y/2 - 1 .. y/2 + 2; plane zp + 2 on its way (pc; pe: the column
-    // beyond the warp's edge, lanes 0 and 31).  The other coarse cell of a fine cell is the
-    // previous one for even cells and the next one for odd cells, or its weight is 0.
-    constexpr int Q = R / 2 + 2;
-    float h0[Q][2], h1[Q][2], pc[Q], pe[Q];
+    // the lane's two columns, rows y/2 - 1 .. y/2 + 2; plane zp + 2 on its way in cplane, zeros outside the
+    // level.  The other coarse cell of a fine cell is the previous one for even cells and the next
+    // one for odd cells, or its weight is 0.
+    constexpr int Q = kCoarse3;
+    float h0[Q][2], h1[Q][2];
     const int cx = x >> 1, cy = y >> 1;  // arithmetic shifts: y may be negative
-    const int xe = lane == 0 ? cx - 1 : cx + 1;
+    float* const crow = cplane + warp * Q * kCoarseW3;  // a row: the column before the warp's, its 32, the one behind
     auto fetch_coarse = [&](int Z) {
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
             const int Y = cy - 1 + q;
-            pc[q] = pe[q] = 0.f;
-            if (Z >= 0 && Z < a.ncz && Y >= 0 && Y < a.ncy) {
-                const float* p = a.cu + ((int64_t)Z * a.ncy + Y) * a.cp;
-                if (cx >= 0 && cx < a.ncx) pc[q] = p[cx];
-                if ((lane == 0 || lane == 31) && xe >= 0 && xe < a.ncx) pe[q] = p[xe];
+            const bool in = Z >= 0 && Z < a.ncz && Y >= 0 && Y < a.ncy;
+            const float* p = a.cu + ((int64_t)Z * a.ncy + Y) * a.cp;
+            float* to = crow + q * kCoarseW3 + 1 + lane;
+            if (in && cx >= 0 && cx < a.ncx) copy4(to, p + cx);
+            else *to = 0.f;
+            if (lane == 0 || lane == 31) {
+                const int e = lane == 0 ? -1 : 1;
+                if (in && cx + e >= 0 && cx + e < a.ncx) copy4(to + e, p + (cx + e));
+                else to[e] = 0.f;
             }
         }
     };
     auto take_coarse = [&](float (&h)[Q][2]) {
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
-            const float v = pc[q];
-            float cw = __shfl_up_sync(0xffffffffu, v, 1), ce = __shfl_down_sync(0xffffffffu, v, 1);
-            if (lane == 0) cw = pe[q];
-            if (lane == 31) ce = pe[q];
-            h[q][0] = fmaf(wx0, cw - v, v);
-            h[q][1] = fmaf(wx1, ce - v, v);
+            const float* from = crow + q * kCoarseW3 + 1 + lane;
+            const float v = from[0];
+            h[q][0] = fmaf(wx0, from[-1] - v, v);
+            h[q][1] = fmaf(wx1, from[1] - v, v);
         }
     };
     if (UP && a.cu) {
-        const int zp = (Tb - 1) >> 1;
+        const int zp = (Tb >> 1) - 1;  // Tb is even
         fetch_coarse(zp);
+        copies_done();
+        __syncthreads();
         take_coarse(h0);
+        __syncthreads();
         fetch_coarse(zp + 1);
+        copies_done();
+        __syncthreads();
         take_coarse(h1);
-        fetch_coarse(zp + 2);
     }
     const int64_t out_row = (int64_t)z0 * ny + y;  // next output plane, this lane's first cell
     float* odst = a.dst + out_row * a.dp + x;
     Split* odst_d = a.d + out_row * a.pitch_d + x;
     const int64_t ostep = (int64_t)ny * a.dp, ostep_d = (int64_t)ny * a.pitch_d;
     float part[2] = {0.f, 0.f};  // restriction: the even plane's 2 x 2 sums of the two coarse rows
-    int slot = Tb % NS;          // ring slot of plane T
+    int slot = Tb % NS;          // ring slot of plane T (edge rows)
     auto slot_of = [&](int back) { const int q = slot - back; return q < 0 ? q + NS : q; };
+    int slot_b = Tb % NB;        // ring slot of plane T (right-hand sides)
+    auto rhs_of = [&](int back) { const int q = slot_b - back; return own + (q < 0 ? q + NB : q) * kTile3 * kTile3; };
+    // UP: plane z of the correction on its way to dplane
+    auto fetch_d = [&](int z) {
+        if (a.d && !a.d_first && lane_out && z >= z0 && z < z1) {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (rows_out >> r & 1) copy16(dplane + ((row0 + r) * (kTile3 / 2) + lane) * 4, odst_d + r * a.pitch_d);
+        }
+    };
     auto edge_at = [&](int sl, int wr, int which) { return edge + ((sl * kWarps3 + wr) * 2 + which) * kTile3 + 2 * lane; };
 
 #pragma unroll 1
     for (int T = Tb; T <= Te; ++T) {
+        copies_done();    // a thread reads only what it copied itself
         __syncthreads();  // edge rows of the last step are visible, those of the oldest plane are free
 #pragma unroll
         for (int q = 0; q + 1 < NP; ++q)
@@ -310,12 +366,13 @@ __global__ void __launch_bounds__(kWarps3 * 32, 1) k3_leg(const Leg3 a) {
             }
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            w[NP - 1][r][0] = pu[r].x;
-            w[NP - 1][r][1] = col1 ? pu[r].y : 0.f;
-            if (!col1) pb[r].y = 0.f;
-            *reinterpret_cast<float2*>(bring + (slot * kTile3 + row0 + r) * kTile3 + 2 * lane) = pb[r];
+            float2 t = make_float2(0.f, 0.f);
+            if (!ZERO) t = *reinterpret_cast<const float2*>(uplane + (((T & 1) * kTile3 + row0 + r) * kTile3 + 2 * lane));
+            w[NP - 1][r][0] = t.x;
+            w[NP - 1][r][1] = t.y;
         }
         if (T < Te) fetch(T + 1);
+        if (UP) fetch_d(T - S);
         if (UP && a.cu && T < nz) {
             if ((T & 1) && T > Tb) {  // planes (T - 1) / 2 and the next one
 #pragma unroll
@@ -324,8 +381,8 @@ __global__ void __launch_bounds__(kWarps3 * 32, 1) k3_leg(const Leg3 a) {
                     h0[q][1] = h1[q][1];
                 }
                 take_coarse(h1);
-                fetch_coarse(((T - 1) >> 1) + 2);
             }
+            if ((T & 1) == 0) fetch_coarse((T >> 1) + 1);  // a barrier after the last reads of cplane
             int Iz, Jz;
             float wz;
             interp_axis<float>(T, a.g.n0z, k, a.ncz, Iz, Jz, wz);
@@ -366,7 +423,7 @@ __global__ void __launch_bounds__(kWarps3 * 32, 1) k3_leg(const Leg3 a) {
                 iD[0] = itab[mx[0] + mz];
                 iD[1] = itab[mx[1] + mz];
             }
-            const float* bp = bring + (sl * kTile3 + row0) * kTile3 + 2 * lane;
+            const float* bp = rhs_of(s);
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 const int i = (I0 + r) & 1;
@@ -408,6 +465,7 @@ __global__ void __launch_bounds__(kWarps3 * 32, 1) k3_leg(const Leg3 a) {
         {   // the plane that completed all half-sweeps
             const int m = T - S;
             const bool mine = m >= z0 && m < z1;
+            if (UP && a.d && !a.d_first) copies_done();
             if (mine && lane_out) {
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
@@ -417,7 +475,8 @@ __global__ void __launch_bounds__(kWarps3 * 32, 1) k3_leg(const Leg3 a) {
                         Split* q = odst_d + r * a.pitch_d;  // 16-byte aligned, the padding included
                         Split e[2] = {{v0, 0.f}, {v1, 0.f}};
                         if (!a.d_first) {
-                            const float4 t = *reinterpret_cast<const float4*>(q);
+                            const float4 t =
+                                *reinterpret_cast<const float4*>(dplane + ((row0 + r) * (kTile3 / 2) + lane) * 4);
                             e[0] = split_add(Split{t.x, t.y}, v0);
                             e[1] = split_add(Split{t.z, t.w}, v1);
                         }
@@ -442,6 +501,7 @@ __global__ void __launch_bounds__(kWarps3 * 32, 1) k3_leg(const Leg3 a) {
             const int m = T - S - 1;
             if (m >= z0 && m < z1) {
                 const int sl = slot_of(S + 1);
+                const float* bp = rhs_of(S + 1);
                 float2 no = make_float2(0.f, 0.f), so = no;
                 if (warp > 0) no = *reinterpret_cast<const float2*>(edge_at(sl, warp - 1, 1));
                 if (warp + 1 < kWarps3) so = *reinterpret_cast<const float2*>(edge_at(sl, warp + 1, 0));
@@ -451,7 +511,7 @@ __global__ void __launch_bounds__(kWarps3 * 32, 1) k3_leg(const Leg3 a) {
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
                     constexpr int P = UP ? 1 : NP - 2 - S;  // plane T - S - 1 (never used for UP)
-                    const float2 bv = *reinterpret_cast<const float2*>(bring + (sl * kTile3 + row0 + r) * kTile3 + 2 * lane);
+                    const float2 bv = *reinterpret_cast<const float2*>(bp + r * kTile3);
                     const float u0 = w[P][r][0], u1 = w[P][r][1];
                     const float uw = __shfl_up_sync(0xffffffffu, u1, 1), ue = __shfl_down_sync(0xffffffffu, u0, 1);
                     const float n0 = r > 0 ? w[P][r > 0 ? r - 1 : 0][0] : no.x, n1 = r > 0 ? w[P][r > 0 ? r - 1 : 0][1] : no.y;
@@ -489,6 +549,7 @@ __global__ void __launch_bounds__(kWarps3 * 32, 1) k3_leg(const Leg3 a) {
             }
         }
         if (++slot == NS) slot = 0;
+        if (++slot_b == NB) slot_b = 0;
     }
 }
 
@@ -846,11 +907,11 @@ int launch_leg3_one(const Leg3& a, dim3 grid, cudaStream_t st) {
     if (dev >= 0 && dev < 64) {
         std::lock_guard<std::mutex> lk(mu);
         if (!done[dev]) {
-            EMF_CUDA(cudaFuncSetAttribute(k3_leg<S, ZERO, UP>, cudaFuncAttributeMaxDynamicSharedMemorySize, leg3_smem<S>()));
+            EMF_CUDA(cudaFuncSetAttribute(k3_leg<S, ZERO, UP>, cudaFuncAttributeMaxDynamicSharedMemorySize, leg3_smem<S, UP>()));
             done[dev] = true;
         }
     }
-    k3_leg<S, ZERO, UP><<<grid, kWarps3 * 32, leg3_smem<S>(), st>>>(a);
+    k3_leg<S, ZERO, UP><<<grid, kWarps3 * 32, leg3_smem<S, UP>(), st>>>(a);
     EMF_CHECK_LAUNCH();
     return EMFUSE_OK;
 }
