@@ -817,7 +817,7 @@ struct Solver {
             kc[j] = fused ? k : nlev[j];
             Kw = std::max(Kw, kc[j]);
         }
-        // levels run by the wavefront kernels (the others by the coarse tail / reference)
+        // levels run by the wavefront or tile kernels (the others by the coarse tail / reference)
         auto wave = [&](int64_t j, int k) { return fused && k < kc[j]; };
         // level arrays: u and b of every slice and level, rows padded to 128 bytes
         const int64_t align = 128 / (int64_t)sizeof(TV);
@@ -1109,7 +1109,7 @@ struct Solver {
         return EMFUSE_OK;
     }
 
-    // Fused schedule: wavefront DOWN on large levels, one coarse-tail kernel, wavefront UP.
+    // Fused schedule: DOWN legs (wavefronts, below kTileMaxCells tiles), one coarse-tail kernel, UP legs.
     // cont = continue from the previous V-cycle's level-0 result (read from uo).
     int vcycle_fused(bool cont) {
         const int S1 = 2 * rq->opts.nu_pre, S2 = 2 * rq->opts.nu_post;
