@@ -55,3 +55,19 @@ def test_adjoint(dev, shape, sigmas):
     assert np.abs(got["o"].cpu().numpy() - lap).max() <= 1e-4 * max(np.abs(lap).max(), 1e-6 * np.abs(lam).max())
     dk = O.dsmooth_dsigma_z(x, *sigmas)
     assert abs(got["sigma_z"] - dsig) <= 1e-4 * np.abs(alpha * lam * dk).sum()
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), -float("inf")])
+@pytest.mark.parametrize("cell", [(0, 0, 0), (12, 20, 16), (23, 39, 32), (11, 8, 31)])
+def test_values_that_are_not_finite_stay_in_their_support(dev, value, cell):
+    """A tap outside the support never meets them: cells beyond it are what they are without."""
+    I0 = make_stack(24, 40, 33, seed=2).to(dev)
+    sigmas, R = (3.0, 1.0), (3, 9, 9)
+    I0[cell] = 0.0
+    ref = api.emfuse_smooth_z(I0, *sigmas)
+    I0[cell] = value
+    out = api.emfuse_smooth_z(I0, *sigmas)
+    inside = torch.zeros(out.shape, dtype=torch.bool, device=dev)
+    inside[tuple(slice(max(0, c - r), c + r + 1) for c, r in zip(cell, R))] = True
+    assert not torch.isfinite(out[inside]).any()
+    assert torch.equal(out[~inside], ref[~inside])
