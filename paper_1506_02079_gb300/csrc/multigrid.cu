@@ -186,6 +186,11 @@ struct CallPtrs {
 constexpr int kTopTX = 64;
 constexpr int kTopTY = 32;  // 8 cells per thread; the one-cell halo of d is 9 % extra
 
+// The residual pass reaches kTopTY rows beyond a tile's corner: more than an int counts?
+inline bool wide_slice(const TopSlice& G) {
+    return (int64_t)(kTopTY + 1) * std::max(G.nx, G.pitch0) > (int64_t)INT32_MAX;
+}
+
 // MODE 0: d = 0, r = alpha (s - o)          (first residual; also accumulates ||b||^2)
 // MODE 1: d_new = e                          (first correction)
 // MODE 2: d_new = d_old + e                  (later corrections)
@@ -204,10 +209,14 @@ constexpr int kTopTY = 32;  // 8 cells per thread; the one-cell halo of d is 9 %
 // instead.  64 x 2048 x 2048, first and later correction together: 4.93 -> 3.50 ms (ragged batch of
 // 291 M cells 7.04 -> 4.82), the first residual 0.73 -> 0.59.  64 warps per SM hide the loads: at 48
 // warps the split passes take 4.17 ms, at 32 5.69.
+//
+// IX: the type of offsets from a tile's corner, which reach kTopTY rows (halo included) of nx or
+// pitch0 cells beyond it.  int where that fits, which saves the registers that 64 warps per SM
+// need; int64_t for slices of about 2^26 cells a row and more (wide_slice).
 enum : int { kRounded = 0, kExact = 1, kSplit = 2 };
 
-template <class TF, class TV, class To, int MODE, int FORM>
-__global__ void __launch_bounds__(256, MODE == 0 ? 6 : 8)
+template <class TF, class TV, class To, int MODE, int FORM, class IX>
+__global__ void __launch_bounds__(256, sizeof(IX) == 8 ? 4 : (MODE == 0 ? 6 : 8))
 k_top(const TopSlice* __restrict__ top, const int64_t* __restrict__ tile_start, int nslices,
       const int* __restrict__ active, const CallPtrs* __restrict__ call, const SolveState* __restrict__ state,
       TF* __restrict__ dbuf0, TF* __restrict__ dbuf1, AlphaDeg<TF> ad,
@@ -237,8 +246,9 @@ k_top(const TopSlice* __restrict__ top, const int64_t* __restrict__ tile_start, 
     using TS = typename std::conditional<!SPLIT, TF, typename std::conditional<MODE == 1, float, Split>::type>::type;
     __shared__ TS dsm[kTopTY + 2][kTopTX + 2];
     // a thread's 8 cells: columns lane and lane + 32 of rows warp, warp + 8, + 16, + 24, so that a
-    // warp reads and writes whole lines; offsets from the tile's corner fit an int
+    // warp reads and writes whole lines
     const int lane = tid & 31, warp = tid >> 5, nx = G.nx;
+    const IX rowx = nx, row0 = G.pitch0;  // row pitches of the packed buffers and of e and r
     const int64_t corner = G.off + (int64_t)ty0 * nx + tx0, corner0 = (int64_t)ty0 * G.pitch0 + tx0;
     const float *sT = rhs ? rhs + corner : s + corner;
     const To* oT = o + corner;
@@ -266,20 +276,20 @@ k_top(const TopSlice* __restrict__ top, const int64_t* __restrict__ tile_start, 
                 const int lx = lane + 32 * (i & 1), ly = warp + 8 * (i >> 1);
                 sva[i] = ova[i] = 0.f;
                 if (inside(lx, ly)) {
-                    sva[i] = sT[ly * nx + lx];
-                    if (!rhs) ova[i] = float(oT[ly * nx + lx]);
+                    sva[i] = sT[ly * rowx + lx];
+                    if (!rhs) ova[i] = float(oT[ly * rowx + lx]);
                 }
             }
         }
         if (MODE >= 1) {
             // the iterate at a cell (halo included)
             auto iterate = [&](int lx, int ly) -> TF {
-                const TF ev = cvt<TF>(eT[ly * G.pitch0 + lx]);
-                return MODE == 1 ? ev : dT[ly * nx + lx] + ev;
+                const TF ev = cvt<TF>(eT[ly * row0 + lx]);
+                return MODE == 1 ? ev : dT[ly * rowx + lx] + ev;
             };
             auto staged = [&](int lx, int ly, TF v) -> TS {
                 if constexpr (!SPLIT) return v;
-                else if constexpr (MODE == 1) return eT[ly * G.pitch0 + lx];
+                else if constexpr (MODE == 1) return eT[ly * row0 + lx];
                 else return split_of(v);
             };
 #pragma unroll kUnroll
@@ -289,7 +299,7 @@ k_top(const TopSlice* __restrict__ top, const int64_t* __restrict__ tile_start, 
                 if (inside(lx, ly)) {
                     const TF v = iterate(lx, ly);
                     c = staged(lx, ly, v);
-                    nT[ly * nx + lx] = v;
+                    nT[ly * rowx + lx] = v;
                 }
                 dsm[ly + 1][lx + 1] = c;
             }
@@ -309,7 +319,8 @@ k_top(const TopSlice* __restrict__ top, const int64_t* __restrict__ tile_start, 
         for (int i = 0; i < 8; ++i) {
             const int lx = lane + 32 * (i & 1), ly = warp + 8 * (i >> 1);
             if (!inside(lx, ly)) continue;
-            const int x = tx0 + lx, y = ty0 + ly, q = ly * nx + lx;
+            const int x = tx0 + lx, y = ty0 + ly;
+            const IX q = ly * rowx + lx;
             const bool hw = INNER || x > 0, he = INNER || x + 1 < nx, hn = INNER || y > 0, hs = INNER || y + 1 < G.ny;
             const float sv = MODE == 0 ? sva[i % kAhead] : sT[q];
             const float ov = MODE == 0 ? ova[i % kAhead] : (rhs ? 0.f : float(oT[q]));
@@ -321,8 +332,8 @@ k_top(const TopSlice* __restrict__ top, const int64_t* __restrict__ tile_start, 
                     float lo = 0.f;
                     if (hw) lo += ov - float(oT[q - 1]);
                     if (he) lo += ov - float(oT[q + 1]);
-                    if (hn) lo += ov - float(oT[q - nx]);
-                    if (hs) lo += ov - float(oT[q + nx]);
+                    if (hn) lo += ov - float(oT[q - rowx]);
+                    if (hs) lo += ov - float(oT[q + rowx]);
                     bv = fmaf(af, sv, lo);
                 }
                 bbf = fmaf(bv, bv, bbf);
@@ -360,7 +371,7 @@ k_top(const TopSlice* __restrict__ top, const int64_t* __restrict__ tile_start, 
                 else f = ov + cf;
                 outT[q] = f;
             }
-            rT[ly * G.pitch0 + lx] = rv;
+            rT[ly * row0 + lx] = rv;
             const float rf = cvt<float>(rv);
             rrf = fmaf(rf, rf, rrf);
         }
@@ -683,6 +694,7 @@ struct Solver {
     int64_t* d_top_ts = nullptr;
     int64_t top_tiles = 0;
     double top_cells = 0;
+    bool top_wide = false;  // a slice is a wide_slice
     TailArgs<TV> tail{};
     double tail_cells = 0;
     bool fused = true;
@@ -765,6 +777,7 @@ struct Solver {
         Kmax = Kw = 0;
         top_tiles = 0;
         top_cells = tail_cells = 0;
+        top_wide = false;
         tail = TailArgs<TV>{};
         built = false;
     }
@@ -936,6 +949,7 @@ struct Solver {
                               (int)ceil_div(rq->nx[j], kTopTX), S0.pitch, S0.uo, S0.b};
             top_ts[j + 1] = top_ts[j] + (int64_t)top[j].tiles_x * ceil_div(rq->ny[j], kTopTY);
             top_cells += (double)rq->nx[j] * rq->ny[j];
+            top_wide |= wide_slice(top[j]);
         }
         top_tiles = top_ts[n];
         std::vector<int> vkc(kc), vnlev(nlev);
@@ -1167,9 +1181,13 @@ struct Solver {
             ad.s[q].lo = float(double(ad.v[q]) - double(ad.s[q].hi));
         }
         ad.alpha_f = float(rq->alpha);
-        auto launch = [&](auto form_tag) {
-            k_top<TF, TV, To, MODE, decltype(form_tag)::value><<<(unsigned)top_tiles, 256, 0, st>>>(
+        auto launch_as = [&](auto form_tag, auto index) {
+            k_top<TF, TV, To, MODE, decltype(form_tag)::value, decltype(index)><<<(unsigned)top_tiles, 256, 0, st>>>(
                 d_top, d_top_ts, (int)rq->nslices, d_active, d_call, d_state, dbuf[0], dbuf[1], ad, d_norms);
+        };
+        auto launch = [&](auto form_tag) {
+            if (top_wide) launch_as(form_tag, int64_t{});
+            else launch_as(form_tag, int{});
         };
         if constexpr (MODE > 0 && sizeof(TV) < sizeof(TF)) {
             if (form == kExact) launch(std::integral_constant<int, kExact>{});
