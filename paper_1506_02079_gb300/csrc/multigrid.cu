@@ -201,7 +201,7 @@ inline bool wide_slice(const TopSlice& G) {
 // (FP64 when mixed).  Conversions between TV and TF run on the integer pipe (fpconv.cuh).
 //
 // Mixed precision, three forms (FORM): kExact (tolerances below 1e-7) subtracts in FP64 too.
-// Otherwise A d is rounded to FP32 before the subtraction, and large batches (kSplit) need not
+// Otherwise A d is rounded to FP32 before the subtraction, and large slices (kSplit) need not
 // form it in FP64: the tile holds the FP64 values split into two floats (48 bits) and A d is
 // evaluated from those on the FP32 pipe (split.cuh), off by about 2^-46 of the largest value
 // before that rounding.  The iterate itself stays in FP64; what is left for the FP64 pipe is the
@@ -670,11 +670,17 @@ struct Blob {
 template <class TV>
 constexpr double kTileMaxCellsOf = sizeof(TV) == 4 ? 5e6 : 2.5e6;
 
-// Batches of at least so many cells form A d of the correction passes in split form (k_top).  Below,
-// the pass is some 5 % of a solve that latency bounds (8.4 M cells: 88 us in FP64, 70 split, in a
-// solve of 1.4 ms), and FP64 keeps the residual's last bits, which a fit that differentiates
-// differences of neighbouring slices amplifies.
-constexpr double kSplitCells = 1.6e7;
+// Slices of at least so many cells form A d of the correction passes in split form (k_top).  The rule
+// looks at the slice alone, never at its batch: the two forms round about 1 % of the cells of r
+// apart, and a slice's result must be the same whole or in chunks, shards and groups.
+// Above the line the FP64 pipe bounds the pass and split form pays (8 slices of 1024 x 1024: 0.79 ms
+// a solve in FP64, 0.75 split; 64 of 2048 x 2048: 12.5 and 10.9).  Below it latency bounds the
+// solve and the pass is 5 to 8 % of it (64 of 512 x 512: 1.22 and 1.13 ms), which is left to FP64: no
+// bits are given up where little is to be had.  Neither form is further from the 64-bit solution:
+// solves and the gradients of fits (64 x 512 x 512, 20 x 1100 x 1100, 6 x 2048 x 2048, alpha 0.001 and 0.01)
+// have the same errors to three digits.
+constexpr int64_t kSplitCells = 1000000;
+inline bool split_slice(int64_t nx, int64_t ny) { return nx * ny >= kSplitCells; }
 
 template <class TF, class TV>
 struct Solver {
@@ -694,6 +700,11 @@ struct Solver {
     int64_t* d_top_ts = nullptr;
     int64_t top_tiles = 0;
     double top_cells = 0;
+    // the residual tiles of the slices that are split_slice and of the others: prefix sums over
+    // all slices (no tiles for the slices of the other kind), tiles, cells
+    int64_t* d_form_ts[2] = {nullptr, nullptr};
+    int64_t form_tiles[2] = {0, 0};
+    double form_cells[2] = {0, 0};
     bool top_wide = false;  // a slice is a wide_slice
     TailArgs<TV> tail{};
     double tail_cells = 0;
@@ -942,16 +953,26 @@ struct Solver {
         }
         // finest-level (residual kernel) tiling
         std::vector<TopSlice> top(n);
-        std::vector<int64_t> top_ts(n + 1, 0);
+        std::vector<int64_t> top_ts(n + 1, 0), form_ts[2];
+        for (int q = 0; q < 2; ++q) {
+            form_ts[q].assign(n + 1, 0);
+            form_cells[q] = 0;
+        }
         for (int64_t j = 0; j < n; ++j) {
             const LSlice<TV> S0 = table[level_off[j]];
             top[j] = TopSlice{rq->offsets[j], (int)rq->nx[j], (int)rq->ny[j],
                               (int)ceil_div(rq->nx[j], kTopTX), S0.pitch, S0.uo, S0.b};
-            top_ts[j + 1] = top_ts[j] + (int64_t)top[j].tiles_x * ceil_div(rq->ny[j], kTopTY);
-            top_cells += (double)rq->nx[j] * rq->ny[j];
+            const int64_t tiles = (int64_t)top[j].tiles_x * ceil_div(rq->ny[j], kTopTY);
+            const double cells = (double)rq->nx[j] * rq->ny[j];
+            const int split = split_slice(rq->nx[j], rq->ny[j]) ? 1 : 0;
+            top_ts[j + 1] = top_ts[j] + tiles;
+            top_cells += cells;
+            for (int q = 0; q < 2; ++q) form_ts[q][j + 1] = form_ts[q][j] + (q == split ? tiles : 0);
+            form_cells[split] += cells;
             top_wide |= wide_slice(top[j]);
         }
         top_tiles = top_ts[n];
+        for (int q = 0; q < 2; ++q) form_tiles[q] = form_ts[q][n];
         std::vector<int> vkc(kc), vnlev(nlev);
         for (int64_t j = 0; j < n; ++j)
             for (int k = kc[j]; k < nlev[j]; ++k) {
@@ -971,6 +992,7 @@ struct Solver {
             pos_tup[k] = blob.add(levels[k].tup_start);
         }
         const size_t pos_top = blob.add(top), pos_top_ts = blob.add(top_ts);
+        const size_t pos_form[2] = {blob.add(form_ts[0]), blob.add(form_ts[1])};
         const size_t pos_table = blob.add(table), pos_loff = blob.add(level_off);
         const size_t pos_nlev = blob.add(vnlev), pos_kc = blob.add(vkc);
         EMF_TRY(ws_desc.alloc_persistent(blob.host.size()));
@@ -987,6 +1009,7 @@ struct Solver {
         }
         d_top = reinterpret_cast<TopSlice*>(dbase + pos_top);
         d_top_ts = reinterpret_cast<int64_t*>(dbase + pos_top_ts);
+        for (int q = 0; q < 2; ++q) d_form_ts[q] = reinterpret_cast<int64_t*>(dbase + pos_form[q]);
         EMF_TRY(ws_norms.alloc_persistent(2 * n * sizeof(double)));
         d_norms = ws_norms.as<double>();
         // active flags of the slices, then the two work counters of the wavefront kernels
@@ -1166,14 +1189,7 @@ struct Solver {
         // d_old in MODE 2) and writes d_new and the output
         const double in_b = rq->rhs ? 4.0 : 4.0 + sizeof(To);
         const double it_b = MODE == 0 ? 0.0 : sizeof(TV) + sizeof(TF) + 4.0 + (MODE == 2 ? sizeof(TF) : 0.0);
-        const double bytes = top_cells * (in_b + it_b + sizeof(TV));
-        // FP64 work of the pass where it bounds it (FP64 iterate, not split): the 5-point operator
-        // on d, three adds and one fma per cell, plus the update d_old + e in MODE 2
-        const bool mixed = sizeof(TV) < sizeof(TF);
-        const int form = MODE == 0 || !mixed ? kRounded
-                                             : (rq->opts.tol < 1e-7 ? kExact : (top_cells >= kSplitCells ? kSplit : kRounded));
-        const double flops = sizeof(TF) == 8 && MODE > 0 && form != kSplit ? top_cells * (MODE == 2 ? 6.0 : 5.0) : 0.0;
-        KernelScope ks(MODE == 0 ? "residual_first" : "residual_update", st, bytes, flops);
+        const double per_cell = in_b + it_b + sizeof(TV);
         AlphaDeg<TF> ad;
         for (int q = 0; q < 5; ++q) {
             ad.v[q] = TF(rq->alpha) + TF(q);
@@ -1181,23 +1197,31 @@ struct Solver {
             ad.s[q].lo = float(double(ad.v[q]) - double(ad.s[q].hi));
         }
         ad.alpha_f = float(rq->alpha);
-        auto launch_as = [&](auto form_tag, auto index) {
-            k_top<TF, TV, To, MODE, decltype(form_tag)::value, decltype(index)><<<(unsigned)top_tiles, 256, 0, st>>>(
-                d_top, d_top_ts, (int)rq->nslices, d_active, d_call, d_state, dbuf[0], dbuf[1], ad, d_norms);
+        auto launch = [&](auto form_tag, const int64_t* ts, int64_t tiles, double cells) -> int {
+            constexpr int FORM = decltype(form_tag)::value;
+            if (tiles == 0) return EMFUSE_OK;
+            // FP64 work of the pass where it bounds it (FP64 iterate, not split): the 5-point
+            // operator on d, three adds and one fma per cell, plus the update d_old + e in MODE 2
+            const double flops = sizeof(TF) == 8 && MODE > 0 && FORM != kSplit ? cells * (MODE == 2 ? 6.0 : 5.0) : 0.0;
+            KernelScope ks(MODE == 0 ? "residual_first" : "residual_update", st, cells * per_cell, flops);
+            auto launch_as = [&](auto index) {
+                k_top<TF, TV, To, MODE, FORM, decltype(index)><<<(unsigned)tiles, 256, 0, st>>>(
+                    d_top, ts, (int)rq->nslices, d_active, d_call, d_state, dbuf[0], dbuf[1], ad, d_norms);
+            };
+            if (top_wide) launch_as(int64_t{});
+            else launch_as(int{});
+            EMF_CHECK_LAUNCH();
+            return EMFUSE_OK;
         };
-        auto launch = [&](auto form_tag) {
-            if (top_wide) launch_as(form_tag, int64_t{});
-            else launch_as(form_tag, int{});
-        };
+        constexpr std::integral_constant<int, kRounded> rounded{};
         if constexpr (MODE > 0 && sizeof(TV) < sizeof(TF)) {
-            if (form == kExact) launch(std::integral_constant<int, kExact>{});
-            else if (form == kSplit) launch(std::integral_constant<int, kSplit>{});
-            else launch(std::integral_constant<int, kRounded>{});
+            if (rq->opts.tol < 1e-7)
+                return launch(std::integral_constant<int, kExact>{}, d_top_ts, top_tiles, top_cells);
+            EMF_TRY(launch(std::integral_constant<int, kSplit>{}, d_form_ts[1], form_tiles[1], form_cells[1]));
+            return launch(rounded, d_form_ts[0], form_tiles[0], form_cells[0]);
         } else {
-            launch(std::integral_constant<int, kRounded>{});
+            return launch(rounded, d_top_ts, top_tiles, top_cells);
         }
-        EMF_CHECK_LAUNCH();
-        return EMFUSE_OK;
     }
 
     int launch_init() {
