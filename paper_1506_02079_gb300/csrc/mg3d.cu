@@ -778,8 +778,9 @@ __global__ void __launch_bounds__(kThreads3) k3_update(D* __restrict__ d, const 
 //
 // A thread marches along z over a chunk of kDefectZ planes of one pixel column, so that the
 // neighbours along z stay in registers; those along y and x are L1 hits of a 32 x 8 tile.  Bound
-// by instruction issue (about 130 per cell): 32 x 1024 x 1024, later passes 509 -> 190 us against
-// FP64 evaluation (bound by that pipe).
+// by instruction issue (about 145 per cell): 32 x 1024 x 1024, a pass 509 -> 201 us against FP64
+// evaluation (bound by that pipe).  The norms' conversions on the integer units: 223 us with the
+// hardware's, which go to the FP64 pipe.
 constexpr int kDefectZ = 16;
 
 template <class D>
@@ -826,7 +827,6 @@ __global__ void __launch_bounds__(kThreads3) k3_defect(const Tin* __restrict__ I
             if (zc > 0) dm = d[q - pz];
             dp = d[q];
         }
-        float rs = 0.f, bs = 0.f;  // FP32 sums of at most kDefectZ squares
         const int ze = min(zc + kDefectZ, nz);
         for (int z = zc; z < ze; ++z, t += sz, q += pz) {
             const bool hd = z > 0, hu = z + 1 < nz;
@@ -864,16 +864,19 @@ __global__ void __launch_bounds__(kThreads3) k3_defect(const Tin* __restrict__ I
                 if (hn) lxy += ip - (float)I0[t - nx];
                 if (hs) lxy += ip - (float)I0[t + nx];
                 const float b = fmaf(alpha, ip, lxy);
-                bs = fmaf(b, b, bs);
+                const double bd = f2d_ieee(b);
+                bb = fma(bd, bd, bb);
             }
-            if (SPLIT || FIRST) rs = fmaf(r, r, rs);
+            // squares in FP64: in FP32 they leave its range (1e-23, 1e19) long before r and b do
+            if (SPLIT || FIRST) {
+                const double rd = f2d_ieee(r);
+                rr = fma(rd, rd, rr);
+            }
             r0[q] = r;
             out[t] = o;
             im = ip;
             ip = in;
         }
-        rr += f2d_ieee(rs);
-        bb += f2d_ieee(bs);
     }
     block_sum2(rr, bb, sums);
 }
