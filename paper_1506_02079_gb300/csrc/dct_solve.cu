@@ -194,7 +194,9 @@ int fft_error(const char* what, cufftResult r) {
     return r == CUFFT_ALLOC_FAILED ? EMFUSE_ENOMEM : EMFUSE_ECUDA;
 }
 
-// Tables of a plan, formed in FP64 on the host and copied before the plan is handed out.
+// Tables of a plan, formed in FP64 on the host and on the device before the plan is handed out:
+// callers on any stream may use it next, and a copy from pageable memory may return before it has
+// reached the device, so it is waited for.  On a stream of its own, which waits for nothing else.
 template <class T>
 int make_tables(FftPlans& p, int64_t nx, int64_t ny, int64_t nz, bool z) {
     using C = typename Fft<T>::C;
@@ -235,7 +237,13 @@ int make_tables(FftPlans& p, int64_t nx, int64_t ny, int64_t nz, bool z) {
         }
     }
     EMF_TRY(p.tables.alloc_persistent(host.size()));
-    EMF_CUDA(cudaMemcpy(p.tables.as<char>(), host.data(), host.size(), cudaMemcpyHostToDevice));
+    cudaStream_t up = nullptr;
+    EMF_CUDA(cudaStreamCreateWithFlags(&up, cudaStreamNonBlocking));
+    cudaError_t e = cudaMemcpyAsync(p.tables.as<char>(), host.data(), host.size(), cudaMemcpyHostToDevice, up);
+    const cudaError_t es = cudaStreamSynchronize(up);
+    cudaStreamDestroy(up);
+    if (e == cudaSuccess) e = es;
+    EMF_CUDA(e);
     return EMFUSE_OK;
 }
 
