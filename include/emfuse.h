@@ -247,8 +247,9 @@ int emfuse_autotune_result(emfuse_tune_entry* out, int max_entries);
  *   s, o, f     device float32, nslices dense slices of ny x nx (uniform batch).
  *   precision   EMFUSE_PREC_FP32 or EMFUSE_PREC_FP64 (transforms and scaling in that type).
  * Temporaries: a copy of the slices and their half spectra (about 1 and 1 times the slices, in
- * the chosen type), from the library's pool; cuFFT plans and the tables of a size are cached per
- * size, batch and precision until emfuse_release_cache().  Asynchronous on `stream`.
+ * the chosen type) and cuFFT's work area, from the library's pool; cuFFT plans and the tables of a
+ * size are cached per size, batch and precision until emfuse_release_cache().  Asynchronous on
+ * `stream`; calls of one size may run at the same time on several streams.
  */
 int emfuse_screened_poisson_dct(const float* s, const float* o, float* f, int64_t nslices, int64_t nx,
                                 int64_t ny, double alpha, int precision, void* stream);
@@ -270,9 +271,10 @@ int emfuse_screened_poisson_dct(const float* s, const float* o, float* f, int64_
  *   alpha       > 0 (finite).
  *   precision   EMFUSE_PREC_FP32 or EMFUSE_PREC_FP64 (transforms and scaling in that type).
  * Temporaries: two copies of the stack and its half spectrum (about 3 times the stack's cells
- * in the chosen type), from the library's pool, plus cuFFT's work area;
+ * in the chosen type), cuFFT's work area and 32 MB for cuBLAS, from the library's pool;
  * EMFUSE_ENOMEM when they do not fit.  The cuFFT plan (per shape and precision) and the
- * cuBLAS handle are cached until emfuse_release_cache().  Asynchronous on `stream`.
+ * cuBLAS handle are cached until emfuse_release_cache().  Asynchronous on `stream`; calls may run
+ * at the same time on several streams.
  */
 int emfuse_smooth_gradient_domain(const void* in, int dt, float* out, int64_t nx, int64_t ny, int64_t nz,
                                   double alpha, int precision, void* stream);

@@ -178,7 +178,8 @@ struct FftPlans {
     cufftHandle fwd = 0, inv = 0;  // none for 1 x 1 slices
     DeviceBuffer tables;           // DctTables, then the z transform's matrix and eigenvalues
     size_t rot_x = 0, lam_y = 0, lam_x = 0, z_mat = 0, z_lam = 0;  // byte offsets
-    std::mutex mu;  // held around cufftSetStream + exec: one plan, calls on several streams
+    size_t work = 0;               // bytes of the transforms' work area, which each call brings
+    std::mutex mu;  // held around cufftSetStream, cufftSetWorkArea and exec: one plan, several callers
     ~FftPlans() {
         if (fwd) cufftDestroy(fwd);
         if (inv) cufftDestroy(inv);
@@ -265,15 +266,18 @@ int get_plans(int64_t nx, int64_t ny, int64_t n, bool z, std::shared_ptr<FftPlan
         long long dims[2] = {(long long)ny, (long long)nx};
         long long* d = rank == 1 ? dims + 1 : dims;
         const long long rdist = nx * ny, cdist = ny * (nx / 2 + 1);
-        size_t work = 0;
+        size_t work[2] = {0, 0};
         cufftResult r = cufftCreate(&p->fwd);
+        if (r == CUFFT_SUCCESS) r = cufftSetAutoAllocation(p->fwd, 0);
         if (r == CUFFT_SUCCESS)
-            r = cufftMakePlanMany64(p->fwd, rank, d, nullptr, 1, rdist, nullptr, 1, cdist, Fft<T>::kR2C, n, &work);
+            r = cufftMakePlanMany64(p->fwd, rank, d, nullptr, 1, rdist, nullptr, 1, cdist, Fft<T>::kR2C, n, &work[0]);
         if (r != CUFFT_SUCCESS) return fft_error("forward plan", r);
         r = cufftCreate(&p->inv);
+        if (r == CUFFT_SUCCESS) r = cufftSetAutoAllocation(p->inv, 0);
         if (r == CUFFT_SUCCESS)
-            r = cufftMakePlanMany64(p->inv, rank, d, nullptr, 1, cdist, nullptr, 1, rdist, Fft<T>::kC2R, n, &work);
+            r = cufftMakePlanMany64(p->inv, rank, d, nullptr, 1, cdist, nullptr, 1, rdist, Fft<T>::kC2R, n, &work[1]);
         if (r != CUFFT_SUCCESS) return fft_error("inverse plan", r);
+        p->work = std::max(work[0], work[1]);
     }
     EMF_TRY((make_tables<T>(*p, nx, ny, n, z)));
     g_fft[key] = p;
@@ -281,10 +285,11 @@ int get_plans(int64_t nx, int64_t ny, int64_t n, bool z, std::shared_ptr<FftPlan
     return EMFUSE_OK;
 }
 
-// forward / inverse transform of the batch on stream st (the plan's lock orders callers on
-// different streams; the transforms themselves run asynchronously)
+// forward / inverse transform of the batch on stream st, in the caller's work area (p.work bytes).
+// Transforms of one plan run asynchronously and at the same time on several streams, so a work area of
+// the plan's own would be shared by them; the lock covers what the plan holds until they are queued.
 template <class T>
-int fft_run(FftPlans& p, T* v, typename Fft<T>::C* spec, int64_t n, bool forward, cudaStream_t st) {
+int fft_run(FftPlans& p, T* v, typename Fft<T>::C* spec, void* work, int64_t n, bool forward, cudaStream_t st) {
     if (!p.fwd) {
         k_single<T, typename Fft<T>::C><<<grid_of(n), 256, 0, st>>>(v, spec, n, forward ? 1 : 0);
         EMF_CHECK_LAUNCH();
@@ -292,6 +297,7 @@ int fft_run(FftPlans& p, T* v, typename Fft<T>::C* spec, int64_t n, bool forward
     }
     std::lock_guard<std::mutex> lk(p.mu);
     cufftResult r = cufftSetStream(forward ? p.fwd : p.inv, st);
+    if (r == CUFFT_SUCCESS && work) r = cufftSetWorkArea(forward ? p.fwd : p.inv, work);
     if (r == CUFFT_SUCCESS) r = forward ? Fft<T>::fwd(p.fwd, v, spec) : Fft<T>::inv(p.inv, spec, v);
     return r == CUFFT_SUCCESS ? EMFUSE_OK : fft_error(forward ? "forward transform" : "inverse transform", r);
 }
@@ -309,7 +315,9 @@ template <class T>
 int dct_filter(FftPlans& p, T* v, typename Fft<T>::C* spec, int64_t nx, int64_t ny, int64_t n, double alpha, bool z,
                const char* name, cudaStream_t st) {
     using C = typename Fft<T>::C;
-    EMF_TRY((fft_run<T>(p, v, spec, n, true, st)));
+    DeviceBuffer work;
+    EMF_TRY(work.alloc(p.work, st));
+    EMF_TRY((fft_run<T>(p, v, spec, work.as<void>(), n, true, st)));
     {
         const char* t = p.tables.as<char>();
         DctTables<T, C> tab;
@@ -324,7 +332,7 @@ int dct_filter(FftPlans& p, T* v, typename Fft<T>::C* spec, int64_t nx, int64_t 
             T(1.0 / ((double)nx * (double)ny)), (int)nx, (int)ny, n);
         EMF_CHECK_LAUNCH();
     }
-    return fft_run<T>(p, v, spec, n, false, st);
+    return fft_run<T>(p, v, spec, work.as<void>(), n, false, st);
 }
 
 template <class T>
@@ -367,8 +375,10 @@ int dct_solve(const float* s, const float* o, float* f, int64_t n, int64_t nx, i
 // slices are permuted into the transform's order before the first and back after the second, in
 // the passes that convert the input and add the result to it.
 
-// cuBLAS handles, one per device, kept until emfuse_release_cache (the lock orders callers on
-// different streams around cublasSetStream + GEMM)
+// cuBLAS handles, one per device, kept until emfuse_release_cache.  As with the transforms, a call
+// brings its own workspace (the handle's would be shared by GEMMs on several streams), and the lock
+// covers cublasSetStream, cublasSetWorkspace and the GEMM's launch.
+constexpr size_t kBlasWorkspace = (size_t)32 << 20;  // what cuBLAS itself takes on this architecture
 struct BlasHandle {
     cublasHandle_t h = nullptr;
     std::mutex mu;
@@ -423,10 +433,11 @@ struct Gemm<double> {
 // matrix C[k][z] read column-major is C^T.  Forward: Y = X C^T (Y[k][p] = sum_z C[k][z] x[z][p]);
 // inverse: Y = X C (Y[z][p] = sum_k C[k][z] x[k][p]).
 template <class T>
-int z_transform(BlasHandle& b, const T* x, const T* cmat, T* y, int64_t P, int64_t nz, bool inverse,
+int z_transform(BlasHandle& b, void* work, const T* x, const T* cmat, T* y, int64_t P, int64_t nz, bool inverse,
                 cudaStream_t st) {
     std::lock_guard<std::mutex> lk(b.mu);
-    cublasStatus_t s = cublasSetStream(b.h, st);
+    cublasStatus_t s = cublasSetStream(b.h, st);  // also resets the handle's workspace
+    if (s == CUBLAS_STATUS_SUCCESS) s = cublasSetWorkspace(b.h, work, kBlasWorkspace);
     if (s == CUBLAS_STATUS_SUCCESS) s = Gemm<T>::run(b.h, inverse ? CUBLAS_OP_T : CUBLAS_OP_N, P, nz, x, cmat, y);
     if (s != CUBLAS_STATUS_SUCCESS) {
         set_error("cuBLAS GEMM of the z transform failed (cublasStatus " + std::to_string((int)s) + ")");
@@ -444,7 +455,8 @@ int gd_smooth(const Tin* in, float* out, int64_t nx, int64_t ny, int64_t nz, dou
     std::shared_ptr<BlasHandle> blas;
     EMF_TRY((get_plans<T>(nx, ny, nz, true, plans)));
     EMF_TRY(get_blas(blas));
-    DeviceBuffer x, y, spec;
+    DeviceBuffer x, y, spec, work;
+    EMF_TRY(work.alloc(kBlasWorkspace, st));
     EMF_TRY(x.alloc((size_t)N * sizeof(T), st));
     EMF_TRY(y.alloc((size_t)N * sizeof(T), st));
     EMF_TRY(spec.alloc((size_t)(nz * ny * (nx / 2 + 1)) * sizeof(C), st));
@@ -455,9 +467,9 @@ int gd_smooth(const Tin* in, float* out, int64_t nx, int64_t ny, int64_t nz, dou
                                                                           nz * ny);
         EMF_CHECK_LAUNCH();
     }
-    EMF_TRY(z_transform<T>(*blas, x.as<T>(), cmat, y.as<T>(), P, nz, false, st));
+    EMF_TRY(z_transform<T>(*blas, work.as<void>(), x.as<T>(), cmat, y.as<T>(), P, nz, false, st));
     EMF_TRY((dct_filter<T>(*plans, y.as<T>(), spec.as<C>(), nx, ny, nz, alpha, true, "gd_scale", st)));
-    EMF_TRY(z_transform<T>(*blas, y.as<T>(), cmat, x.as<T>(), P, nz, true, st));
+    EMF_TRY(z_transform<T>(*blas, work.as<void>(), y.as<T>(), cmat, x.as<T>(), P, nz, true, st));
     {
         KernelScope ks("gd_out", st, (double)N * (sizeof(Tin) + sizeof(T) + 4.0));
         k_extract<T, Tin><<<row_grid(nz * ny), row_threads(nx), 0, st>>>(x.as<T>(), in, out, (int)nx, (int)ny, nz * ny);

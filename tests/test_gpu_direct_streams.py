@@ -1,5 +1,6 @@
 """The direct solvers on streams other than the default one: the first call of a size, which forms
-the plan's tables, gives what later calls on other streams give."""
+the plan's tables, gives what later calls on other streams give, and calls of one size that run at
+the same time on several streams (one plan, one handle) give what they give one after another."""
 import numpy as np
 import pytest
 import torch
@@ -37,3 +38,22 @@ def test_first_call_of_a_size(dev, shape, precision):
         torch.cuda.synchronize()
         assert torch.equal(first, again)
         assert torch.equal(first, call())
+
+
+# sides with large prime factors, whose transforms need a work area, and a GEMM with few columns
+@pytest.mark.parametrize("shape", [(6, 509, 521), (40, 127, 131), (3, 1, 100003), (900, 5, 7)])
+@pytest.mark.parametrize("precision", [api.PREC_FP32, api.PREC_FP64])
+def test_same_size_on_several_streams_at_once(dev, shape, precision):
+    rng = np.random.default_rng(22)
+    side = [torch.cuda.Stream() for _ in range(4)]
+    s = [torch.from_numpy(rng.uniform(0, 255, size=shape).astype(np.float32)).to(dev) for _ in side]
+    o = [(0.9 * a + 10).contiguous() for a in s]
+    serial = [api.emfuse_screened_poisson_dct(s[q], o[q], 0.01, precision) for q in range(len(side))]
+    serial3 = [api.emfuse_smooth_gradient_domain(s[q], 0.05, precision) for q in range(len(side))]
+    torch.cuda.synchronize()
+    got = [on(side[q % 4], lambda: api.emfuse_screened_poisson_dct(s[q % 4], o[q % 4], 0.01, precision)) for q in range(24)]
+    got3 = [on(side[q % 4], lambda: api.emfuse_smooth_gradient_domain(s[q % 4], 0.05, precision)) for q in range(24)]
+    torch.cuda.synchronize()
+    for q in range(24):
+        assert torch.equal(got[q], serial[q % 4])
+        assert torch.equal(got3[q], serial3[q % 4])
