@@ -132,14 +132,15 @@ k_scale(C* __restrict__ spec, DctTables<T, C> tab, const T* __restrict__ lam_z, 
             const T px = b.x * A.x - b.y * A.y, py = b.x * A.y + b.y * A.x;
             const T qx = b.x * B.x - b.y * B.y, qy = b.x * B.y + b.y * B.x;
             const T l0 = tab.lam_x[l], l1 = l == 0 ? T(0) : tab.lam_x[nx - l];
-            const T h = T(0.5) * norm * num;
+            // the gain first: alpha times a sum may leave the type's range where the gain does not
+            const T h = T(0.5) * norm;
             // P + Q* = (px + qx, py - qy), Q + P* its conjugate; P - Q* = (px - qx, py + qy),
             // Q - P* = (qx - px, qy + py)
             const T sx = px + qx, sy = py - qy, dx = px - qx, dy = py + qy;
-            const T x00 = h * (a.x * sx - a.y * sy) / (y0 + l0);
-            const T x10 = k == 0 ? T(0) : h * (-a.x * sy - a.y * sx) / (y1 + l0);
-            const T x01 = l == 0 ? T(0) : -h * (a.x * dy + a.y * dx) / (y0 + l1);
-            const T x11 = k == 0 || l == 0 ? T(0) : h * (a.y * dy - a.x * dx) / (y1 + l1);
+            const T x00 = h * (num / (y0 + l0)) * (a.x * sx - a.y * sy);
+            const T x10 = k == 0 ? T(0) : h * (num / (y1 + l0)) * (-a.x * sy - a.y * sx);
+            const T x01 = l == 0 ? T(0) : -h * (num / (y0 + l1)) * (a.x * dy + a.y * dx);
+            const T x11 = k == 0 || l == 0 ? T(0) : h * (num / (y1 + l1)) * (a.y * dy - a.x * dx);
             // a b* and a* b*
             const T ux = a.x * b.x + a.y * b.y, uy = a.y * b.x - a.x * b.y;
             const T wx = a.x * b.x - a.y * b.y, wy = -(a.x * b.y + a.y * b.x);
