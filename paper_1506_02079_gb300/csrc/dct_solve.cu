@@ -19,7 +19,7 @@
 // slices); permutation, scaling and extraction are the kernels below.  All passes are bound by
 // memory (64 B per cell in FP32, the two transforms' passes included).  Transforming the mirror
 // extension (2ny x 2nx) instead, four times the points, took 0.99 ms for 16 x 1024 x 1024 in FP32
-// where this takes 0.26 ms (3-D gradient domain, 32 x 1024 x 1024 uint8: 2.25 -> 0.66 ms).
+// where this takes 0.25 ms (3-D gradient domain, 32 x 1024 x 1024 uint8: 2.25 -> 0.63 ms).
 #include <cuda_runtime.h>
 #include <cublas_v2.h>
 #include <cufft.h>
@@ -128,6 +128,7 @@ k_scale(C* __restrict__ spec, DctTables<T, C> tab, const T* __restrict__ lam_z, 
         C* rk = spec + (j * ny + k) * cols;
         C* rr = spec + (j * ny + r) * cols;
         const C a = tab.rot_y[k];
+        const T hx = T(0.5) * norm * a.x, hy = T(0.5) * norm * a.y;
         const T lz = lam_z ? lam_z[j] : T(0);
         const T num = lam_z ? -lz : alpha;
         const T y0 = alpha + lz + tab.lam_y[k], y1 = k == 0 ? T(1) : alpha + lz + tab.lam_y[ny - k];
@@ -136,18 +137,17 @@ k_scale(C* __restrict__ spec, DctTables<T, C> tab, const T* __restrict__ lam_z, 
             const T px = b.x * A.x - b.y * A.y, py = b.x * A.y + b.y * A.x;
             const T qx = b.x * B.x - b.y * B.y, qy = b.x * B.y + b.y * B.x;
             const T l0 = tab.lam_x[l], l1 = l == 0 ? T(0) : tab.lam_x[nx - l];
-            // the gain first: alpha times a sum may leave the type's range where the gain does not
-            const T h = T(0.5) * norm;
             // P + Q* = (px + qx, py - qy), Q + P* its conjugate; P - Q* = (px - qx, py + qy),
             // Q - P* = (qx - px, qy + py)
             const T sx = px + qx, sy = py - qy, dx = px - qx, dy = py + qy;
-            const T x00 = h * (num / (y0 + l0)) * (a.x * sx - a.y * sy);
-            const T x10 = k == 0 ? T(0) : h * (num / (y1 + l0)) * (-a.x * sy - a.y * sx);
-            const T x01 = l == 0 ? T(0) : -h * (num / (y0 + l1)) * (a.x * dy + a.y * dx);
-            const T x11 = k == 0 || l == 0 ? T(0) : h * (num / (y1 + l1)) * (a.y * dy - a.x * dx);
-            // a b* and a* b*
-            const T ux = a.x * b.x + a.y * b.y, uy = a.y * b.x - a.x * b.y;
-            const T wx = a.x * b.x - a.y * b.y, wy = -(a.x * b.y + a.y * b.x);
+            // the gain first: alpha times a sum may leave the type's range where the gain does not
+            const T x00 = num / (y0 + l0) * (a.x * sx - a.y * sy);
+            const T x10 = k == 0 ? T(0) : num / (y1 + l0) * (-a.x * sy - a.y * sx);
+            const T x01 = l == 0 ? T(0) : -num / (y0 + l1) * (a.x * dy + a.y * dx);
+            const T x11 = k == 0 || l == 0 ? T(0) : num / (y1 + l1) * (a.y * dy - a.x * dx);
+            // a b* and a* b*, times norm / 2
+            const T ux = hx * b.x + hy * b.y, uy = hy * b.x - hx * b.y;
+            const T wx = hx * b.x - hy * b.y, wy = -(hx * b.y + hy * b.x);
             const T e = x00 - x11, g = -(x10 + x01);
             C o0;
             o0.x = wx * e - wy * g;
@@ -323,12 +323,10 @@ inline dim3 row_blocks(int64_t rows, int64_t cells) {
 
 // v -> cosine coefficients scaled -> v, in the transform's order (lam_z: see k_scale)
 template <class T>
-int dct_filter(FftPlans& p, T* v, typename Fft<T>::C* spec, int64_t nx, int64_t ny, int64_t n, double alpha, bool z,
+int dct_filter(FftPlans& p, T* v, typename Fft<T>::C* spec, void* work, int64_t nx, int64_t ny, int64_t n, double alpha, bool z,
                const char* name, cudaStream_t st) {
     using C = typename Fft<T>::C;
-    DeviceBuffer work;
-    EMF_TRY(work.alloc(p.work, st));
-    EMF_TRY((fft_run<T>(p, v, spec, work.as<void>(), n, true, st)));
+    EMF_TRY((fft_run<T>(p, v, spec, work, n, true, st)));
     {
         const char* t = p.tables.as<char>();
         DctTables<T, C> tab;
@@ -343,7 +341,7 @@ int dct_filter(FftPlans& p, T* v, typename Fft<T>::C* spec, int64_t nx, int64_t 
             T(1.0 / ((double)nx * (double)ny)), (int)nx, (int)ny, n);
         EMF_CHECK_LAUNCH();
     }
-    return fft_run<T>(p, v, spec, work.as<void>(), n, false, st);
+    return fft_run<T>(p, v, spec, work, n, false, st);
 }
 
 template <class T>
@@ -353,18 +351,23 @@ int dct_solve(const float* s, const float* o, float* f, int64_t n, int64_t nx, i
     if (nx == 1) std::swap(nx, ny);  // a column is a row in memory
     std::shared_ptr<FftPlans> plans;
     EMF_TRY((get_plans<T>(nx, ny, n, false, plans)));
-    DeviceBuffer v, spec;
-    EMF_TRY(v.alloc((size_t)(n * nx * ny) * sizeof(T), st));
-    EMF_TRY(spec.alloc((size_t)(n * ny * (nx / 2 + 1)) * sizeof(C), st));
+    // one allocation: the spectra (first, for their alignment), the slices, cuFFT's work area
+    const size_t nspec = round_up(n * ny * (nx / 2 + 1) * (int64_t)sizeof(C), 256);
+    const size_t nv = round_up(n * nx * ny * (int64_t)sizeof(T), 256);
+    DeviceBuffer tmp;
+    EMF_TRY(tmp.alloc(nspec + nv + plans->work, st));
+    C* const spec = tmp.as<C>();
+    T* const v = reinterpret_cast<T*>(tmp.as<char>() + nspec);
+    void* const work = plans->work ? tmp.as<char>() + nspec + nv : nullptr;
     {
         KernelScope ks("dct_permute", st, (double)n * nx * ny * (8.0 + sizeof(T)));
-        k_permute<T, float><<<row_blocks(n * ny, nx), row_threads(nx), 0, st>>>(s, o, v.as<T>(), (int)nx, (int)ny, n * ny);
+        k_permute<T, float><<<row_blocks(n * ny, nx), row_threads(nx), 0, st>>>(s, o, v, (int)nx, (int)ny, n * ny);
         EMF_CHECK_LAUNCH();
     }
-    EMF_TRY((dct_filter<T>(*plans, v.as<T>(), spec.as<C>(), nx, ny, n, alpha, false, "dct_scale", st)));
+    EMF_TRY((dct_filter<T>(*plans, v, spec, work, nx, ny, n, alpha, false, "dct_scale", st)));
     {
         KernelScope ks("dct_extract", st, (double)n * nx * ny * (4.0 + 4.0 + sizeof(T)));
-        k_extract<T, float><<<row_blocks(n * ny, nx), row_threads(nx), 0, st>>>(v.as<T>(), o, f, (int)nx, (int)ny, n * ny);
+        k_extract<T, float><<<row_blocks(n * ny, nx), row_threads(nx), 0, st>>>(v, o, f, (int)nx, (int)ny, n * ny);
         EMF_CHECK_LAUNCH();
     }
     // the temporaries go back to the pool stream-ordered; the caller's stream orders f
@@ -466,24 +469,29 @@ int gd_smooth(const Tin* in, float* out, int64_t nx, int64_t ny, int64_t nz, dou
     std::shared_ptr<BlasHandle> blas;
     EMF_TRY((get_plans<T>(nx, ny, nz, true, plans)));
     EMF_TRY(get_blas(blas));
-    DeviceBuffer x, y, spec, work;
-    EMF_TRY(work.alloc(kBlasWorkspace, st));
-    EMF_TRY(x.alloc((size_t)N * sizeof(T), st));
-    EMF_TRY(y.alloc((size_t)N * sizeof(T), st));
-    EMF_TRY(spec.alloc((size_t)(nz * ny * (nx / 2 + 1)) * sizeof(C), st));
+    // one allocation: the spectra (first, for their alignment), the stack twice, and one work area for
+    // the transforms and the GEMMs, which follow one another on the stream
+    const size_t nspec = round_up(nz * ny * (nx / 2 + 1) * (int64_t)sizeof(C), 256);
+    const size_t nstack = round_up(N * (int64_t)sizeof(T), 256);
+    DeviceBuffer tmp;
+    EMF_TRY(tmp.alloc(nspec + 2 * nstack + std::max(plans->work, kBlasWorkspace), st));
+    C* const spec = tmp.as<C>();
+    T* const x = reinterpret_cast<T*>(tmp.as<char>() + nspec);
+    T* const y = reinterpret_cast<T*>(tmp.as<char>() + nspec + nstack);
+    void* const work = tmp.as<char>() + nspec + 2 * nstack;
     const T* cmat = reinterpret_cast<const T*>(plans->tables.as<char>() + plans->z_mat);
     {
         KernelScope ks("gd_permute", st, (double)N * (sizeof(Tin) + sizeof(T)));
-        k_permute<T, Tin><<<row_blocks(nz * ny, nx), row_threads(nx), 0, st>>>(in, nullptr, x.as<T>(), (int)nx, (int)ny,
+        k_permute<T, Tin><<<row_blocks(nz * ny, nx), row_threads(nx), 0, st>>>(in, nullptr, x, (int)nx, (int)ny,
                                                                           nz * ny);
         EMF_CHECK_LAUNCH();
     }
-    EMF_TRY(z_transform<T>(*blas, work.as<void>(), x.as<T>(), cmat, y.as<T>(), P, nz, false, st));
-    EMF_TRY((dct_filter<T>(*plans, y.as<T>(), spec.as<C>(), nx, ny, nz, alpha, true, "gd_scale", st)));
-    EMF_TRY(z_transform<T>(*blas, work.as<void>(), y.as<T>(), cmat, x.as<T>(), P, nz, true, st));
+    EMF_TRY(z_transform<T>(*blas, work, x, cmat, y, P, nz, false, st));
+    EMF_TRY((dct_filter<T>(*plans, y, spec, work, nx, ny, nz, alpha, true, "gd_scale", st)));
+    EMF_TRY(z_transform<T>(*blas, work, y, cmat, x, P, nz, true, st));
     {
         KernelScope ks("gd_out", st, (double)N * (sizeof(Tin) + sizeof(T) + 4.0));
-        k_extract<T, Tin><<<row_blocks(nz * ny, nx), row_threads(nx), 0, st>>>(x.as<T>(), in, out, (int)nx, (int)ny, nz * ny);
+        k_extract<T, Tin><<<row_blocks(nz * ny, nx), row_threads(nx), 0, st>>>(x, in, out, (int)nx, (int)ny, nz * ny);
         EMF_CHECK_LAUNCH();
     }
     return EMFUSE_OK;
