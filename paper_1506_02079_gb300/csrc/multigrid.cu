@@ -667,6 +667,12 @@ struct Blob {
 // tiles / wavefronts, FP32: 0.26 M cells 25 / 53, 1 M 40 / 64, 4.2 M 66 / 73, 5.2 M 73 / 71,
 // 9.5 M (odd width) 105 / 85, 17 M 163 / 119.  FP64 (the FP64 pipe bounds the recomputed cells):
 // 1.2 M 277 / 375, 4.7 M 860 / 770.
+//
+// A tile costs the same however little of it lies in the level, so the tiles' own cells, halos included,
+// are counted too: at most twice as many (a level of large slices has 1.4 to 1.5 times its cells).  Slices of
+// few rows, us per solve with every level below the line by tiles / with the line at 2 / at 1.4
+// times: 1 x 2,000,000 9777 / 3425 / 3260, 8 x 500,000 1998 / 1363 / 1288, 20 of 1 x 200,000 18660 / 5285 /
+// 5094; 1000 of 65 x 65 1662 / 1615 / 1581, which the line at 1.4 would buy with slower 2000 x 2000 slices.
 template <class TV>
 constexpr double kTileMaxCellsOf = sizeof(TV) == 4 ? 5e6 : 2.5e6;
 
@@ -929,8 +935,10 @@ struct Solver {
                     std::vector<int64_t>& ts = leg == 0 ? L.tdn_start : L.tup_start;
                     ts.push_back(0);
                     for (const auto& S : L.wsl) ts.push_back(ts.back() + ceil_div(S.nx, ox) * ceil_div(S.ny, oy));
+                    const double area = (double)(ox + 2 * L.hx[leg]) * (oy + 2 * L.hy[leg]);
+                    if ((double)ts.back() * area > 2.0 * kTileMaxCells) L.tile = false;
                 }
-                continue;  // no wavefront items, no tensor maps
+                if (L.tile) continue;  // no wavefront items, no tensor maps
             }
             for (const auto& S : L.wsl) {
                 L.item_start.push_back(L.item_start.back() + (int64_t)S.fstrips * ceil_div(S.ny, L.ch));
