@@ -194,13 +194,51 @@ struct AxisParams {
 // index divisions in 64 bits, now 26 us along x and 24 along y (R = 3), 32 along z (R = 7, two sets of taps).
 // Bound by instruction issue at small radii (80 % of the slots), with 10 us of memory traffic.
 
+// Rows narrower than so many cells are taken as one line of cells (FLAT): a lane finds the row of its
+// cells by divisions of its own, where a warp to a row would leave most lanes without one.  The whole
+// smoothing (sigma 4 and 5, float), a warp to a row / as one line: 40 x 5001 x 3 353 / 199 us, 40 x 1000 x 20
+// 139 / 115, x 48 151 / 137, x 63 156 / 142.
+constexpr int kAxisFlat = 64;
+
 // Along x: a warp makes 128 cells of a row, a lane every 32nd; the taps' loads hit L1.
-template <class Tin>
+template <class Tin, bool FLAT>
 __global__ void __launch_bounds__(256)
 axis_x_kernel(const Tin* __restrict__ in, float* __restrict__ out, int nx, int64_t rows, int64_t pitch_in, int64_t pitch_out,
               const float* __restrict__ pre, const float* __restrict__ post, AxisParams prm) {
     const int lane = threadIdx.x & 31;
-    const int64_t segs = (nx + 127) / 128, warps = (int64_t)gridDim.x * 8;
+    const int64_t warps = (int64_t)gridDim.x * 8;
+    if constexpr (FLAT) {
+        const int64_t cells = rows * nx;
+        for (int64_t item = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); item * 128 < cells; item += warps) {
+            int c[4];
+            const Tin* src[4];
+            float* dst[4];
+            float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int64_t q = item * 128 + lane + 32 * t, row = index_div(q, nx);
+                c[t] = q < cells ? (int)(q - row * nx) : nx + kAxisMaxRadius;  // past the end: no tap lies inside
+                src[t] = in + row * pitch_in;
+                dst[t] = out + row * pitch_out + c[t];
+            }
+            for (int d = -prm.R; d <= prm.R; ++d) {
+                const float w = prm.w[kAxisGroup - 1 + d + prm.R];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    const int e = c[t] + d;
+                    if (e < 0 || e >= nx) continue;
+                    float v = float(src[t][e]);
+                    if (pre) v *= pre[e];
+                    acc[t] = fmaf(w, v, acc[t]);
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                if (c[t] < nx) *dst[t] = post ? acc[t] * post[c[t]] : acc[t];
+        }
+        return;
+    }
+    const int64_t segs = (nx + 127) / 128;
     for (int64_t item = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); item < segs * rows; item += warps) {
         const int64_t row = index_div(item, segs);
         const int x0 = (int)(item - row * segs) * 128, x = x0 + lane;
@@ -247,7 +285,8 @@ axis_x_kernel(const Tin* __restrict__ in, float* __restrict__ out, int nx, int64
 // the axis from one read of their common inputs, so R = 7 reads 22 values for 8 cells, not 120.
 // The groups of a column run next to each other and share their halos in L1 and L2.  `outer` counts
 // the other of the two axes.  DUAL: out = post * (w taps) + post2 * (w2 taps), from the same reads.
-template <bool DUAL>
+// The z passes take a plane as one row.
+template <bool DUAL, bool FLAT>
 __global__ void __launch_bounds__(256, DUAL ? 3 : 4)
 axis_yz_kernel(const float* __restrict__ in, float* __restrict__ out, int nx, int len, int64_t stride, int64_t outer,
                int64_t outer_stride, const float* __restrict__ pre, const float* __restrict__ post,
@@ -256,11 +295,23 @@ axis_yz_kernel(const float* __restrict__ in, float* __restrict__ out, int nx, in
     constexpr int G = kAxisGroup;
     const int lane = threadIdx.x & 31, R = prm.R;
     const int64_t groups = (len + G - 1) / G, segs = (nx + 31) / 32, warps = (int64_t)gridDim.x * 8;
-    for (int64_t item = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); item < groups * segs * outer; item += warps) {
-        const int64_t col = index_div(item, groups), q = index_div(col, segs);
-        const int c0 = (int)(item - col * groups) * G;
-        const int x = (int)(col - q * segs) * 32 + lane;
-        if (x >= nx) continue;
+    const int64_t items = FLAT ? (groups * nx * outer + 31) / 32 : groups * segs * outer;
+    for (int64_t item = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); item < items; item += warps) {
+        int64_t q;
+        int c0, x;
+        if constexpr (FLAT) {
+            const int64_t t = item * 32 + lane, col = index_div(t, nx);
+            q = index_div(col, groups);
+            c0 = (int)(col - q * groups) * G;
+            x = (int)(t - col * nx);
+            if (q >= outer) continue;
+        } else {
+            const int64_t col = index_div(item, groups);
+            q = index_div(col, segs);
+            c0 = (int)(item - col * groups) * G;
+            x = (int)(col - q * segs) * 32 + lane;
+            if (x >= nx) continue;
+        }
         const float* p = in + (q * outer_stride + x + (int64_t)(c0 - R) * stride);
         float acc[G], acc2[G];
 #pragma unroll
@@ -368,11 +419,19 @@ static int launch_axis_x(const void* in, int dt, float* out, int64_t nx, int64_t
     EMF_TRY(axis_params(w, &prm));
     const int64_t rows = ny * nz;
     KernelScope ks("smooth_axis", st, (double)nx * rows * ((dt == EMFUSE_U8 ? 1.0 : 4.0) + 4.0));
-    const unsigned blocks = axis_blocks(ceil_div(nx, 128) * rows);
-    if (dt == EMFUSE_U8)
-        axis_x_kernel<uint8_t><<<blocks, 256, 0, st>>>((const uint8_t*)in, out, (int)nx, rows, pin, nx, pre, post, prm);
-    else
-        axis_x_kernel<float><<<blocks, 256, 0, st>>>((const float*)in, out, (int)nx, rows, pin, nx, pre, post, prm);
+    const bool flat = nx < kAxisFlat;
+    const unsigned blocks = axis_blocks(flat ? ceil_div(nx * rows, 128) : ceil_div(nx, 128) * rows);
+    auto launch = [&](auto tin, auto flat_tag) {
+        using Tin = decltype(tin);
+        axis_x_kernel<Tin, decltype(flat_tag)::value><<<blocks, 256, 0, st>>>((const Tin*)in, out, (int)nx, rows, pin, nx, pre,
+                                                                               post, prm);
+    };
+    auto launch_as = [&](auto tin) {
+        if (flat) launch(tin, std::true_type{});
+        else launch(tin, std::false_type{});
+    };
+    if (dt == EMFUSE_U8) launch_as(uint8_t{});
+    else launch_as(float{});
     EMF_CHECK_LAUNCH();
     return EMFUSE_OK;
 }
@@ -384,16 +443,23 @@ static int launch_axis_yz(const float* in, float* out, int64_t nx, int64_t ny, i
     AxisParams prm{}, prm2{};
     EMF_TRY(axis_params(w, &prm));
     if (w2) EMF_TRY(axis_params(*w2, &prm2));
+    KernelScope ks("smooth_axis", st, 8.0 * nx * ny * nz);
+    if (axis == 2 && nx * ny <= INT32_MAX) {  // a plane as one row
+        nx *= ny;
+        ny = 1;
+    }
     const int64_t len = axis == 1 ? ny : nz, stride = axis == 1 ? nx : nx * ny;
     const int64_t outer = axis == 1 ? nz : ny, outer_stride = axis == 1 ? nx * ny : nx;
-    KernelScope ks("smooth_axis", st, 8.0 * nx * ny * nz);
-    const unsigned blocks = axis_blocks(ceil_div(len, kAxisGroup) * ceil_div(nx, 32) * outer);
-    if (w2)
-        axis_yz_kernel<true><<<blocks, 256, 0, st>>>(in, out, (int)nx, (int)len, stride, outer, outer_stride, pre, post, post2, prm,
-                                                     prm2);
-    else
-        axis_yz_kernel<false><<<blocks, 256, 0, st>>>(in, out, (int)nx, (int)len, stride, outer, outer_stride, pre, post, nullptr,
-                                                      prm, prm2);
+    const int64_t groups = ceil_div(len, kAxisGroup);
+    const bool flat = nx < kAxisFlat && !w2;
+    const unsigned blocks = axis_blocks(flat ? ceil_div(groups * nx * outer, 32) : groups * ceil_div(nx, 32) * outer);
+    auto launch = [&](auto dual_tag, auto flat_tag) {
+        axis_yz_kernel<decltype(dual_tag)::value, decltype(flat_tag)::value><<<blocks, 256, 0, st>>>(
+            in, out, (int)nx, (int)len, stride, outer, outer_stride, pre, post, post2, prm, prm2);
+    };
+    if (w2) launch(std::true_type{}, std::false_type{});
+    else if (flat) launch(std::false_type{}, std::true_type{});
+    else launch(std::false_type{}, std::false_type{});
     EMF_CHECK_LAUNCH();
     return EMFUSE_OK;
 }
