@@ -507,7 +507,16 @@ int smooth_stack(const void* in, int dt, float* out, int64_t nx, int64_t ny, int
     const size_t esz = dt == EMFUSE_U8 ? 1 : 4;
     const bool tma_ok = Rxy <= 4 && Rz <= 9 && force_path == 0;
     const bool aligned = (pitch * (int64_t)esz) % 16 == 0 && (reinterpret_cast<uintptr_t>(in) & 15) == 0;
-    if (tma_ok && (aligned || (Rxy >= 1 && Rz >= 1))) {
+    const int64_t zin0 = std::max<int64_t>(0, z0 - Rz), zin1 = std::min<int64_t>(nz, z1 + Rz), nzin = zin1 - zin0;
+    // Unaligned rows: packed (below), or by plain loads.  The copy's launch, its memory and the tensor map are
+    // 7 us of host time, which marches of a plane or two over small planes do not earn back (us a call,
+    // packed / plain, float: 1 x 100 x 101 24.9 / 17.4 one after another and 35.8 / 31.2 alone, 1 x 600 x 601 25.4 / 20.3
+    // and 41.2 / 38.2, 1 x 1000 x 1001 26.9 / 26.7 and 48.6 / 47.6, 2 x 600 x 601 26.4 / 25.4 and 43.4 / 47.6, 3 x 300 x 301
+    // 24.6 / 19.2 and 38.6 / 40.4, robust 24.8 / 29.9 and 48.5 / 50.4).  Supports below one cell, which no one
+    // smooths by, have no packed instances.
+    const bool few = nzin <= (rob ? 2 : 3) && nx * ny * nzin <= 400000;
+    const bool packed = !aligned && Rxy >= 1 && Rz >= 1 && !few;
+    if (tma_ok && (aligned || packed)) {
         SmoothTmaCall c{};
         c.prm.Rxy = Rxy;
         c.prm.Rz = Rz;
@@ -531,7 +540,6 @@ int smooth_stack(const void* in, int dt, float* out, int64_t nx, int64_t ny, int
             set_error("could not allocate the device error word");
             return EMFUSE_ECUDA;
         }
-        const int64_t zin0 = std::max<int64_t>(0, z0 - Rz), zin1 = std::min<int64_t>(nz, z1 + Rz);
         const double bytes = (double)nx * ((zin1 - zin0) * (double)esz + (z1 - z0) * 4.0);  // per row
         if (aligned) {
             EMF_TRY(encode_tensor_map_3d(&c.map, in, (int)esz, nx, ny, nz, pitch, kTX + hx + hxr, kTY + 2 * Rxy));
@@ -559,7 +567,7 @@ int smooth_stack(const void* in, int dt, float* out, int64_t nx, int64_t ny, int
         // where smooth_fused_kernel took 2.32 (float 0.29 and 0.45 for 2.52; robust 1.68 for 3.73
         // and 1.95 for 4.06, copy included).  A slab is at most kPackBytes; where not even one
         // tile's rows fit, or there is no memory for it, smooth_fused_kernel still runs.
-        const int64_t ppitch = round_up(nx, 16 / (int64_t)esz), nzin = zin1 - zin0;
+        const int64_t ppitch = round_up(nx, 16 / (int64_t)esz);
         const int64_t row_bytes = nzin * ppitch * (int64_t)esz;
         int64_t rows = std::min<int64_t>(ny, kPackBytes / row_bytes - 2 * Rxy);  // output rows of a slab
         if (rows < ny) rows = rows / kTY * kTY;
@@ -607,7 +615,6 @@ int smooth_stack(const void* in, int dt, float* out, int64_t nx, int64_t ny, int
         prm.kappa2 = kappa * kappa;
         dim3 grid((unsigned)ceil_div(nx, kTX), (unsigned)ceil_div(ny, kTY));
         const int P = 2 * Rz + 1;
-        const int64_t zin0 = std::max<int64_t>(0, z0 - Rz), zin1 = std::min<int64_t>(nz, z1 + Rz);
         KernelScope ks(rob ? "smooth_fused_robust" : "smooth_fused", st,
                        (double)nx * ny * ((zin1 - zin0) * (dt == EMFUSE_U8 ? 1.0 : 4.0) + (z1 - z0) * 4.0));
 #define EMF_SMOOTH_LAUNCH1(PP, RB)                                                             \
@@ -635,8 +642,6 @@ int smooth_stack(const void* in, int dt, float* out, int64_t nx, int64_t ny, int
         return EMFUSE_OK;
     }
     // Three renormalised 1-D passes (x, y over the needed input planes; then z).
-    const int64_t zin0 = std::max<int64_t>(0, z0 - Rz), zin1 = std::min<int64_t>(nz, z1 + Rz);
-    const int64_t nzin = zin1 - zin0;
     DeviceBuffer t1, t2;
     EMF_TRY(t1.alloc((size_t)(nzin * ny * nx) * sizeof(float), st));
     EMF_TRY(t2.alloc((size_t)(nzin * ny * nx) * sizeof(float), st));
