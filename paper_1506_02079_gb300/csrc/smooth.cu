@@ -166,6 +166,7 @@ k_pack(const T* __restrict__ in, T* __restrict__ out, int nx, int y0, int ny_sla
         const T* src = in + ((z0 + z) * ny + y0 + y) * pitch;
         T* dst = out + row * ppitch;
         if (sizeof(T) == 1) {  // 4 bytes per store; the last store stays inside the padded row
+#pragma unroll 1  // one or two rounds on most rows: unrolled it costs 2 us of 28
             for (int x = 4 * first; x < nx; x += 4 * step) {
                 uint32_t v = 0;
 #pragma unroll
