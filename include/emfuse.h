@@ -288,7 +288,7 @@ int emfuse_smooth_gradient_domain(const void* in, int dt, float* out, int64_t nx
  * opts->nu_pre / nu_post sweeps; opts->first_vcycles FP32 cycles before the first FP64 pass);
  * after every V-cycle d += e, and a pass forms r = -L_z in - A d (d and A d in two floats per
  * value, 48 bits, A d rounded once to FP32 before the subtraction from the FP32-formed -L_z in;
- * everything in FP64 when opts->tol < 1e-7) and writes out = in + d, until ||r|| / ||alpha in + L_xy in|| <= opts->tol
+ * everything in FP64 when opts->tol < 1e-7 or alpha < 1e-5) and writes out = in + d, until ||r|| / ||alpha in + L_xy in|| <= opts->tol
  * or opts->max_vcycles V-cycles.  The host reads the residual norm after every pass (the call
  * returns when out is final).  Other opts fields are ignored.
  *   in      device, nz x ny x nx dense [z][y][x], uint8 (dt = EMFUSE_U8) or float32.

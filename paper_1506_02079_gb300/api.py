@@ -378,7 +378,7 @@ def emfuse_smooth_gradient_domain_mg(stack: torch.Tensor, alpha: float, opts: So
                                      allow_noconv: bool = False):
     """The 3-D gradient-domain smoothing by multigrid on the stack (Sec. 3 "Alternate Solutions"):
     FP32 V-cycles on the 7-point operator with defect correction to opts.tol (two floats per value,
-    FP64 for tol < 1e-7).  ``stack`` CUDA uint8 or float32 [z][y][x].  Returns float32 of the same shape (and with return_stats
+    FP64 for tol < 1e-7 or alpha < 1e-5).  ``stack`` CUDA uint8 or float32 [z][y][x].  Returns float32 of the same shape (and with return_stats
     one dict for the whole stack)."""
     _require_cuda(stack)
     if stack.dim() != 3 or not stack.is_contiguous():

@@ -15,7 +15,7 @@
 //     x + y + z) with nu_pre / nu_post sweeps;
 //   * V-cycles in FP32 on the correction equation, outer defect-correction passes: d += e,
 //     r = -L_z I0 - A d, out = I0 + d, until ||r|| / ||alpha I0 + L_xy I0|| <= tol; d and A d in
-//     two floats per value (48 bits, split.cuh), in FP64 for tol < 1e-7.
+//     two floats per value (48 bits, split.cuh), in FP64 for tol < 1e-7 or alpha < 1e-5.
 //
 // A leg of a level is one pass over memory (k3_leg: the red-black half-sweeps pipelined along z,
 // with the prolongation before or the restriction after them); levels of at most kTail3 cells
@@ -771,7 +771,7 @@ __global__ void __launch_bounds__(kThreads3) k3_update(D* __restrict__ d, const 
 // Defect pass on the finest level: r = -L_z I0 - A d (A = alpha I + L, 7-point, Neumann), out =
 // I0 + d; r goes to the level-0 right-hand side (FP32).  sums[0] += ||r||^2; with FIRST (d = 0, not
 // read) also sums[1] += ||alpha I0 + L_xy I0||^2.  Three forms of d: Split (two floats, tolerances
-// from 1e-7): A d carries the rounding errors of its sums and product and is rounded once to FP32
+// from 1e-7 and alpha from 1e-5): A d carries the rounding errors of its sums and product and is rounded once to FP32
 // before it is taken from the FP32-formed -L_z I0 (exact for 8-bit input; its own rounding bounds
 // what more bits could add there); double with everything in FP64, -L_z I0 and the subtraction
 // included (smaller tolerances, where that rounding would cap the reachable residual).
@@ -997,7 +997,11 @@ int gd_multigrid(const void* in, int dt, float* out, int64_t nx, int64_t ny, int
         }
     }
     const size_t coarse = all - padded(0), n0p = padded(0);
-    const bool split = opts.tol >= 1e-7;
+    // d and A d in two floats, unless the tolerance or alpha asks for more: 48 bits of 6 + alpha hold alpha
+    // itself to 2^-46 / alpha, which reaches d's smooth part as that share of it.  Root-mean-square error of
+    // 24 x 300 x 301 (0 .. 255) at tol 1e-6, d in FP64 with A d rounded to FP32 / two floats: alpha = 1e-4 1.4e-4 /
+    // 1.4e-4, 1e-5 2.1e-4 / 1.5e-4, 1e-6 1.7e-4 / 6.0e-4.
+    const bool split = opts.tol >= 1e-7 && alpha >= 1e-5;
     // Iterate buffers.  A leg reads one buffer and ends in the other: DOWN u -> v (from u only when
     // a V-cycle continues from the last one), UP v -> u.  The finest level's v is the caller's
     // `out`, which every defect pass rewrites; and between its two legs the finest level's u is
