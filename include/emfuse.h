@@ -92,7 +92,7 @@ typedef struct {
                             power of two in [8, 256].  No effect where the finest level is
                             small enough (about 5 M cells in FP32) to run by tiles.         */
     int autotune;        /* 1: before solving, time complete solves of this batch for
-                            tile_rows in {32, 64, 128, 256} (with nu = (2, 2)), then for
+                            tile_rows in {0, 64, 128, 256} (with nu = (2, 2)), then for
                             (nu_pre, nu_post) in {(1,1), (1,2), (2,1), (2,3), (3,2), (3,3),
                             (3,4), (4,4)} with each of the two fastest tile_rows (fused
                             schedule; nu_pre = 4 runs its DOWN leg in the reference

@@ -1636,11 +1636,13 @@ static int solve_batch_once(const SolveRequest& req, cudaStream_t st) {
 // ---------------------------------------------------------------- autotuner
 // Schedules are compared by the time of a complete solve to the requested tolerance (a
 // schedule with fewer sweeps is cheaper per V-cycle but may need more V-cycles).  The search
-// is staged: rows per work item on the finest level in {32, 64, 128, 256} with nu = (2, 2),
-// then (nu_pre, nu_post) in {(1, 1), (1, 2), (2, 1), (2, 3), (3, 2), (3, 3), (3, 4)} with the best
-// rows (one to four red-black sweeps per leg, all in the fused wavefront kernels).  Each candidate runs twice (the
-// first run builds its plan and captures its graphs) and the second run is timed.  The winner
-// is cached per batch geometry, alpha, precision and tol.
+// is staged: rows per work item on the finest level with nu = (2, 2), the chosen height (wave_rows,
+// tile_rows = 0) first, so that tuning never ends with less than the default, and 64, 128 and 256;
+// then (nu_pre, nu_post) in {(1, 1), (1, 2), (2, 1), (2, 3), (3, 2), (3, 3), (3, 4), (4, 4)} with each of the
+// two fastest heights.  (Where the finest level runs by tiles the heights are the same schedule, and
+// the trials repeat.)  Each candidate runs twice (the first run builds its plan and captures its
+// graphs) and the second run is timed.  The winner is cached per batch geometry, alpha, precision
+// and tol.
 namespace {
 struct TuneKey {
     std::vector<int64_t> geom;
@@ -1733,7 +1735,7 @@ int solve_batch(const SolveRequest& req, cudaStream_t st) {
     };
     // rows per work item (the tile height of a 128-column strip) at nu = (2, 2), then every
     // other sweep count with the two fastest tile heights
-    for (int rows : {32, 64, 128, 256}) EMF_TRY(trial(2, 2, rows));
+    for (int rows : {0, 64, 128, 256}) EMF_TRY(trial(2, 2, rows));
     std::vector<emfuse_tune_entry> by_rows(table);
     std::stable_sort(by_rows.begin(), by_rows.end(), [](const emfuse_tune_entry& x, const emfuse_tune_entry& y) {
         const double a = x.ms < 0 ? 1e300 : x.ms, c = y.ms < 0 ? 1e300 : y.ms;
