@@ -159,6 +159,11 @@ void emfuse_default_opts(emfuse_solve_opts* opts);
  *   sigma_xy, sigma_z >= 0 (0 = no smoothing along that axis).
  *
  * Weights are renormalised over in-stack taps at stack ends and slice edges.
+ * Temporaries from the library's pool, whose idle pages stay mapped until emfuse_release_cache() or
+ * until another allocation of the process needs them: the normalisers; for rows whose byte pitch or base is no multiple
+ * of 16, slabs of at most 512 MB that hold them at an aligned pitch (where there is no memory for
+ * one the rows are read as they are, with the same result); for supports beyond 4 (xy) or 9 (z)
+ * cells three copies of the planes read, in float32.
  * Asynchronous on `stream`.
  */
 int emfuse_smooth_z(const void* in, int dt, float* out, int64_t nx, int64_t ny, int64_t nz,
