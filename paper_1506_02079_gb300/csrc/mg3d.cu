@@ -751,7 +751,7 @@ __device__ __forceinline__ void block_sum2(double a, double b, double* sums) {
         }
         if (l == 0) {
             atomicAdd(&sums[0], a);
-            atomicAdd(&sums[1], b);
+            if (b != 0.0) atomicAdd(&sums[1], b);  // only the first pass has the second sum
         }
     }
 }
@@ -777,7 +777,9 @@ __global__ void __launch_bounds__(kThreads3) k3_update(D* __restrict__ d, const 
 // included (smaller tolerances, where that rounding would cap the reachable residual).
 //
 // A thread marches along z over a chunk of kDefectZ planes of one pixel column, so that the
-// neighbours along z stay in registers; those along y and x are L1 hits of a 32 x 8 tile.  Bound
+// neighbours along z stay in registers; those along y and x are L1 hits of a 32 x 8 tile.  A block takes
+// `per` such items, several where the stack has few planes: with one each, the sums' atomics
+// bounded the pass (a call on 1 x 2048 x 2048: 168 us, now 95).  Bound
 // by instruction issue (about 145 per cell): 32 x 1024 x 1024, a pass 509 -> 201 us against FP64
 // evaluation (bound by that pipe).  The norms' conversions on the integer units: 223 us with the
 // hardware's, which go to the FP64 pipe.
@@ -808,15 +810,17 @@ __device__ __forceinline__ float split_apply7(Split a, Split c, Split w, Split e
 template <class Tin, class D, bool FIRST>
 __global__ void __launch_bounds__(kThreads3) k3_defect(const Tin* __restrict__ I0, const D* __restrict__ d,
                                                        float* __restrict__ r0, float* __restrict__ out, int nx, int ny,
-                                                       int nz, int pitch, float alpha, Adeg3<D> adeg,
-                                                       double* __restrict__ sums) {
+                                                       int nz, int pitch, unsigned items, unsigned per, float alpha,
+                                                       Adeg3<D> adeg, double* __restrict__ sums) {
     constexpr bool SPLIT = std::is_same<D, Split>::value;
     const unsigned tx = (unsigned)((nx - 1) / 32 + 1), ty = (unsigned)((ny - 1) / 8 + 1);
-    const unsigned tile = blockIdx.x / tx, chunk = tile / ty;
-    const int x = int(blockIdx.x - tile * tx) * 32 + (threadIdx.x & 31);
-    const int y = int(tile - chunk * ty) * 8 + (threadIdx.x >> 5), zc = int(chunk) * kDefectZ;
+    const unsigned end = min((blockIdx.x + 1) * per, items);
     double rr = 0.0, bb = 0.0;
-    if (x < nx && y < ny) {
+    for (unsigned item = blockIdx.x * per; item < end; ++item) {
+        const unsigned tile = item / tx, chunk = tile / ty;
+        const int x = int(item - tile * tx) * 32 + (threadIdx.x & 31);
+        const int y = int(tile - chunk * ty) * 8 + (threadIdx.x >> 5), zc = int(chunk) * kDefectZ;
+        if (x >= nx || y >= ny) continue;
         const int64_t sz = (int64_t)nx * ny, pz = (int64_t)pitch * ny;
         int64_t t = ((int64_t)zc * ny + y) * nx + x, q = ((int64_t)zc * ny + y) * pitch + x;
         const bool hw = x > 0, he = x + 1 < nx, hn = y > 0, hs = y + 1 < ny;
@@ -1036,7 +1040,9 @@ int gd_multigrid(const void* in, int dt, float* out, int64_t nx, int64_t ny, int
             const double n0 = (double)nx * ny * nz;
             KernelScope ks("gd3_defect", st, n0 * ((dt == EMFUSE_U8 ? 1.0 : 4.0) + (first ? 0.0 : 8.0) + 8.0),
                            first || split ? 0.0 : n0 * 8.0);
-            const unsigned grid = (unsigned)(ceil_div(nx, 32) * ceil_div(ny, 8) * ceil_div(nz, kDefectZ));
+            const unsigned items = (unsigned)(ceil_div(nx, 32) * ceil_div(ny, 8) * ceil_div(nz, kDefectZ));
+            const unsigned per = (unsigned)std::max<int64_t>(1, kDefectZ / nz);
+            const unsigned grid = (items - 1) / per + 1;
             auto run = [&](auto tin, auto dd, auto first_tag) {
                 using Tin = decltype(tin);
                 using D = decltype(dd);
@@ -1051,7 +1057,7 @@ int gd_multigrid(const void* in, int dt, float* out, int64_t nx, int64_t ny, int
                     }
                 }
                 k3_defect<Tin, D, decltype(first_tag)::value><<<grid, kThreads3, 0, st>>>(
-                    (const Tin*)in, (const D*)d, lev[0].b, out, (int)nx, (int)ny, (int)nz, lev[0].pitch, af, adeg,
+                    (const Tin*)in, (const D*)d, lev[0].b, out, (int)nx, (int)ny, (int)nz, lev[0].pitch, items, per, af, adeg,
                     sums.as<double>());
             };
             auto run_d = [&](auto tin) {
