@@ -497,7 +497,7 @@ def run_gpu(args):
             sm[label] = {"ms": ms_s, "value": voxels / (ms_s * 1e-3), "unit": "voxels/s", "gbs": gbs,
                          "hbm_frac": gbs / measured_hbm_peak()[0]}
         extras["smoothing"] = sm
-        # the second next row: the direct FFT solve of the same 64 solves (mirror extension,
+        # the second next row: the direct solve of the same 64 solves (cosine transforms by
         # cuFFT) against the multigrid solve alone, and their largest difference
         s_c2 = api.emfuse_smooth_z(I0, 1.0, 3.0)
         sol = {}
@@ -560,7 +560,7 @@ def run_gpu(args):
         del base, s_rgb
         torch.cuda.empty_cache()
         # the fourth next row: phase 1 as the 3-D gradient-domain problem of the earlier method
-        # (exact, one 3-D FFT of the mirror-extended stack) beside the Gaussian smoothing above;
+        # (exact, cosine transforms of the slices between two z transforms) beside the Gaussian smoothing above;
         # alpha = 0.1 damps per-slice offsets over about 1 / sqrt(alpha) ~ 3 slices, like sigma_z = 3
         gd, outs = {}, {}
         for label, prec in (("fp32", api.PREC_FP32), ("fp64", api.PREC_FP64)):

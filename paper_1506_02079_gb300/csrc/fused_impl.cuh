@@ -23,8 +23,10 @@
 //
 // Rows of a step: see `step` in k_wave for its three bodies.  Running the steps at the top of a
 // chunk by the same range-check-free bodies as the rest, and strips of any width by cached
-// stencils, took level 0 of 64 x 2048 x 2048 from 0.556 to 0.507 ms per UP leg (6.9 TB/s), of 96
-// ragged slices (291 M cells) from 1.08 to 0.66 ms (7.1 TB/s).
+// stencils, took level 0 of 64 x 2048 x 2048 from 0.556 to 0.507 ms per UP leg, of 96 ragged slices
+// (291 M cells) from 1.08 to 0.66 ms, on average over solves in whose last V-cycles most slices have
+// converged.  With every slice at work: 0.59 ms (5.9 TB/s, 0.87 of the copy rate) and 0.81 ms (5.7); DOWN
+// legs 0.54 to 0.56 (5.3) and 0.76 (5.2).
 //
 // Levels whose larger side is <= 64 are run by one CTA per slice: tail_warps.cuh (FP32),
 // tail_cells.cuh (FP64).
@@ -94,7 +96,8 @@ constexpr int kWaveWarps = 4;  // warps (strips) per CTA
 __host__ __device__ constexpr int wmod(int a, int w) { return ((a % w) + w) % w; }
 
 // CTAs per SM the register budget is sized for: the register window grows with the sweeps (S + 3
-// row pairs) and FP64 windows take twice the registers.
+// row pairs) and FP64 windows take twice the registers (the continuing DOWN leg in FP64 at S = 4, once a
+// solve, spills 24 bytes).
 template <class T, int S>
 struct WaveOcc { static constexpr int value = (sizeof(T) == 4 && S <= 4) ? 4 : 2; };
 

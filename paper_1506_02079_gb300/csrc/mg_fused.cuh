@@ -105,28 +105,6 @@ __device__ __forceinline__ Coef<T> make_coef(const AxisCoef<T>& ax, const AxisCo
     return c;
 }
 
-// The stencil of a cell on an interior row (ay = {1, 1, 1}) with D and 1/D taken from a
-// per-column cache (d, id) computed by make_coef on such a row: the same values make_coef
-// returns, without recomputing the diagonal and its reciprocal.
-template <class T>
-__device__ __forceinline__ Coef<T> interior_row_coef(const AxisCoef<T>& ax, int k, T sk, T d, T id) {
-    Coef<T> c;
-    if (k == 0) {
-        c.cw = ax.gm;
-        c.ce = ax.gp;
-        c.cn = T(1);
-        c.cs = T(1);
-    } else {
-        c.cw = sk * (T(1) * ax.gm);
-        c.ce = sk * (T(1) * ax.gp);
-        c.cn = sk * (ax.w * T(1));
-        c.cs = sk * (ax.w * T(1));
-    }
-    c.D = d;
-    c.iD = id;
-    return c;
-}
-
 // Rows whose axis_coef is {1, 1, 1} (see axis_coef).
 __device__ __forceinline__ bool interior_row(int r, int n, int k) {
     return k == 0 ? (r >= 1 && r + 1 < n) : (r >= 1 && r + 2 < n);

@@ -207,8 +207,9 @@ inline bool wide_slice(const TopSlice& G) {
 // before that rounding.  The iterate itself stays in FP64; what is left for the FP64 pipe is the
 // update d_old + e of MODE 2 (the first correction has none), and the pass is bound by memory
 // instead.  64 x 2048 x 2048, first and later correction together: 4.93 -> 3.50 ms (ragged batch of
-// 291 M cells 7.04 -> 4.82), the first residual 0.73 -> 0.59.  64 warps per SM hide the loads: at 48
-// warps the split passes take 4.17 ms, at 32 5.69.
+// 291 M cells 7.04 -> 4.82), the first residual 0.73 -> 0.59.  64 warps per SM hide the loads (at
+// 32 registers, where MODE 1 in split form spills 16 bytes): at 48 warps the split passes take 4.17 ms, at 32
+// 5.69.
 //
 // IX: the type of offsets from a tile's corner, which reach kTopTY rows (halo included) of nx or
 // pitch0 cells beyond it.  int where that fits, which saves the registers that 64 warps per SM

@@ -19,7 +19,8 @@
 // (another diagonal) and on rows of partial cells (the level's table).
 // 16 slices of 64 x 64, 2 + 2 sweeps: 23 us per launch, 60 x 60 25, 16 x 16 17; passes
 // over cells in shared memory (tail_cells.cuh) take 33, 33 and 19, with stencils formed in every pass
-// they took 137.  FP64 keeps those: one warp's FP64 instructions take 16 cycles each, so few warps
+// they took 137.  Both blocks' state at once (the 64- and 32-levels') is a few registers more than the 128 of
+// 512 threads: 88 bytes a thread spill, written and read between the legs.  FP64 keeps those: one warp's FP64 instructions take 16 cycles each, so few warps
 // with every second lane idle are slower there (170 against 80 us).
 #pragma once
 #include <cuda_runtime.h>
@@ -118,7 +119,6 @@ __device__ __forceinline__ T tail_interp(const TailLevel<T>& L, const T* c, int 
 // The block's part of a level: R rows of C columns per lane (R = 4, C = 2 or R = 2, C = 1).
 template <class T, int R, int C>
 struct TailBlock {
-    static constexpr int kCols = 32 * C;
     TailLevel<T> L;
     T u[R][C], b[R][C], id[R][C];
     ColCoefs<T> col[C];
@@ -243,7 +243,7 @@ struct TailBlock {
     }
 };
 
-// The CTA's shared memory (dynamic: more than 48 KB in FP64).
+// The CTA's shared memory.
 template <class T>
 struct alignas(16) TailShared {
     TailTables<T> tab;

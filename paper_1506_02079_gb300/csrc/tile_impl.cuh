@@ -23,7 +23,8 @@
 //
 // Bound by latency and barriers (two CTAs of 16 warps per SM): one 128 x 128 level of 16 slices
 // takes 8 us where the wavefront kernel's march took 25; 64 registers hold the 32 values and
-// their neighbours, taller warps would leave one CTA per SM.
+// their neighbours (the UP leg's coarse rows spill 52 bytes while it loads), taller warps would leave
+// one CTA per SM.
 #pragma once
 #include <cuda_runtime.h>
 
