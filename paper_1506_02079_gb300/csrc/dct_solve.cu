@@ -116,7 +116,10 @@ struct DctTables {
 // X(., nx) = 0,
 //     row k:       a* b* ((X(k, l) - X(ny-k, nx-l)) - i (X(ny-k, l) + X(k, nx-l)))
 //     row ny - k:  a  b* ((X(k, l) + X(ny-k, nx-l)) + i (X(ny-k, l) - X(k, nx-l)))
-template <class T, class C>
+// GAIN: the gain first, for an alpha whose product with a coefficient leaves the type's range where the
+// gain does not.  Not needed for 1e-20 <= alpha <= 1e20 (coefficients of 2^29 cells a side and values of
+// 1e-10 .. 1e10 stay in FP32's range there), and 3 % slower in FP64 (20 x 400 x 700 217 -> 223 us).
+template <class T, class C, bool GAIN>
 __global__ void __launch_bounds__(256)
 k_scale(C* __restrict__ spec, DctTables<T, C> tab, const T* __restrict__ lam_z, T alpha, T norm, int nx, int ny,
         int64_t nslices) {
@@ -128,10 +131,10 @@ k_scale(C* __restrict__ spec, DctTables<T, C> tab, const T* __restrict__ lam_z, 
         C* rk = spec + (j * ny + k) * cols;
         C* rr = spec + (j * ny + r) * cols;
         const C a = tab.rot_y[k];
-        const T hx = T(0.5) * norm * a.x, hy = T(0.5) * norm * a.y;
         const T lz = lam_z ? lam_z[j] : T(0);
         const T num = lam_z ? -lz : alpha;
         const T y0 = alpha + lz + tab.lam_y[k], y1 = k == 0 ? T(1) : alpha + lz + tab.lam_y[ny - k];
+        const T h = GAIN ? T(0.5) * norm : T(0.5) * norm * num;
         for (int l = first_of_row(); l < cols; l += row_step()) {
             const C A = rk[l], B = rr[l], b = tab.rot_x[l];
             const T px = b.x * A.x - b.y * A.y, py = b.x * A.y + b.y * A.x;
@@ -140,14 +143,17 @@ k_scale(C* __restrict__ spec, DctTables<T, C> tab, const T* __restrict__ lam_z, 
             // P + Q* = (px + qx, py - qy), Q + P* its conjugate; P - Q* = (px - qx, py + qy),
             // Q - P* = (qx - px, qy + py)
             const T sx = px + qx, sy = py - qy, dx = px - qx, dy = py + qy;
-            // the gain first: alpha times a sum may leave the type's range where the gain does not
-            const T x00 = num / (y0 + l0) * (a.x * sx - a.y * sy);
-            const T x10 = k == 0 ? T(0) : num / (y1 + l0) * (-a.x * sy - a.y * sx);
-            const T x01 = l == 0 ? T(0) : -num / (y0 + l1) * (a.x * dy + a.y * dx);
-            const T x11 = k == 0 || l == 0 ? T(0) : num / (y1 + l1) * (a.y * dy - a.x * dx);
-            // a b* and a* b*, times norm / 2
-            const T ux = hx * b.x + hy * b.y, uy = hy * b.x - hx * b.y;
-            const T wx = hx * b.x - hy * b.y, wy = -(hx * b.y + hy * b.x);
+            auto scaled = [&](T sum, T den) {
+                if constexpr (GAIN) return h * (num / den) * sum;
+                else return h * sum / den;
+            };
+            const T x00 = scaled(a.x * sx - a.y * sy, y0 + l0);
+            const T x10 = k == 0 ? T(0) : scaled(-a.x * sy - a.y * sx, y1 + l0);
+            const T x01 = l == 0 ? T(0) : -scaled(a.x * dy + a.y * dx, y0 + l1);
+            const T x11 = k == 0 || l == 0 ? T(0) : scaled(a.y * dy - a.x * dx, y1 + l1);
+            // a b* and a* b*
+            const T ux = a.x * b.x + a.y * b.y, uy = a.y * b.x - a.x * b.y;
+            const T wx = a.x * b.x - a.y * b.y, wy = -(a.x * b.y + a.y * b.x);
             const T e = x00 - x11, g = -(x10 + x01);
             C o0;
             o0.x = wx * e - wy * g;
@@ -309,8 +315,8 @@ int fft_run(FftPlans& p, T* v, typename Fft<T>::C* spec, void* work, int64_t n, 
 
 // Threads and blocks of a pass over `rows` rows of `cells` cells: a block per row while the rows
 // fill the chip (loops beyond that), several blocks to a row where they do not.  Two rows of 200,000
-// cells in FP64: 2.67 ms with a block per row, in which
-// each thread takes 800 cells one after another, 0.28 with the chip filled (FP32 0.63 and 0.10).
+// cells in FP64: 2.67 ms with a block per row, in which each thread takes 800 cells one after another,
+// 0.28 with the chip filled (FP32 0.63 and 0.10).
 inline unsigned row_threads(int64_t cells) {
     return (unsigned)std::min<int64_t>(256, round_up(std::max<int64_t>(cells, 1), 32));
 }
@@ -336,7 +342,9 @@ int dct_filter(FftPlans& p, T* v, typename Fft<T>::C* spec, void* work, int64_t 
         tab.lam_x = reinterpret_cast<const T*>(t + p.lam_x);
         const int64_t cols = nx / 2 + 1;
         KernelScope ks(name, st, (double)n * ny * cols * 2.0 * sizeof(C));
-        k_scale<T, C><<<row_blocks(n * (ny / 2 + 1), cols), row_threads(cols), 0, st>>>(
+        const bool gain = !z && (alpha < 1e-20 || alpha > 1e20);
+        auto* kernel = gain ? k_scale<T, C, true> : k_scale<T, C, false>;
+        kernel<<<row_blocks(n * (ny / 2 + 1), cols), row_threads(cols), 0, st>>>(
             spec, tab, z ? reinterpret_cast<const T*>(t + p.z_lam) : nullptr, T(alpha),
             T(1.0 / ((double)nx * (double)ny)), (int)nx, (int)ny, n);
         EMF_CHECK_LAUNCH();
